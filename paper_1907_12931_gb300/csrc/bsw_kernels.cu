@@ -437,15 +437,15 @@ __device__ __forceinline__ unsigned long long inter_pair(const Batch &B, const P
 // ------------------------------------------ two rows per instruction (8-bit)
 //
 // The 8-bit class pairs without N bases take rows in pairs: rows i and i+1 sit
-// in the low and high halves of s16x2 registers, row i+1 one column behind
+// in the high and low halves of s16x2 registers, row i+1 one column behind
 // (step s computes cells (i, s) and (i+1, s-1)), so every DPX instruction of
 // the cell update (Eq. 2, Eq. 3's affine gaps) advances two cells.  Row i+1
 // takes its diagonal H(i, s-2) and its E(i+1, s-1) from row i's registers;
 // only row i+1's results go back to the slot column, slot s-1 <- {H(i+1, s-2),
 // E(i+2, s-1)}, so a pass reads each slot once and writes it once for two
 // rows.  The row selector in bits 0-15 of slot s picks byte q_s of row i's
-// profile for the low half and byte 4 + q_{s-1} (row i+1's profile) for the
-// high half, both sign-extended, so one byte permute gives both scores.
+// profile for the high half and byte 4 + q_{s-1} (row i+1's profile) for the
+// low half, both sign-extended, so one byte permute gives both scores.
 //
 // Row i+1's band depends on row i's rule-c trims, which are known only after
 // row i ends.  Its left end is found before the packed loop starts: row i
@@ -461,6 +461,93 @@ __device__ __forceinline__ unsigned long long inter_pair(const Batch &B, const P
 // row i+1 run after the loop, once L is known, reading the slot past row i's
 // end as a row-by-row pass does (a value an earlier row left there, read when
 // the band grows past the previous row's end).
+// What bounds it: the ALU pipe (DPX instructions, permutes) and issue
+// together, at the 12 warps an SM's shared memory holds, so the step is built
+// to issue little and to use the FMA pipe where that costs no instruction:
+//   - what E and F open from, max(0, M - o - e), is one half-precision
+//     subtraction on the whole numbers' bit patterns: a half with bits v in
+//     [0, 2047] is v * 2^-24 exactly (subnormal, or the first normal binade
+//     with the same spacing), .sat clamps at zero, and a negative M (two's
+//     complement, so a NaN pattern down to -1023) comes out as +0, as .sat
+//     turns NaN into +0.
+//   - row i sits in the high half and row i+1 in the low one, so that the
+//     16 bits that go back to a slot are one sum, H * 256 + E, of which
+//     H * 256 is the row key's product as well.
+//   - H and E come out of the slot word by one permute each, which also moves
+//     row i's values into row i+1's half.
+//   - L is settled once per block of steps: nothing to do but note the block
+//     when its last cell of row i is positive (the usual case).
+// 4 M pairs of 250 bp reads: 13.56 ms with the clamp on the ALU pipe, byte
+// loads of E, a permute for the store and L tracked by two instructions a
+// step; 10.76 ms so.
+__device__ __forceinline__ uint32_t sub_sat_h2(uint32_t a, uint32_t b)
+{
+    uint32_t d;
+    asm("sub.rn.sat.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+
+// A thread's constants and running values of the row-pair pass: high halves
+// row i, low halves row i + 1.
+struct RpK {
+    uint32_t p0, p1;                        // byte c: score of (t_i, c), (t_{i+1}, c)
+    uint32_t oe_d2, oe_i2, ne_d2, ne_i2;    // o + e; -e
+    uint32_t k8, zm;                        // 2^8 and the zero-diagonal factor 2^7
+};
+struct RpRow {
+    uint32_t hA, hB;                        // H of steps s - 1 and s - 2
+    uint32_t hK;                            // hA * 256
+    uint32_t EN, F;                         // E out of step s - 1; F into step s
+    uint32_t key;                           // row keys H * 256 + column
+    uint32_t j2;                            // s << 16 | s - 1
+    int L;                                  // last column of row i with H > 0, plus 1
+};
+
+// N steps from step s: cells (i, s + k) and (i + 1, s + k - 1).  All N slots
+// are read before the first is written back (step s + k writes slot s + k - 1,
+// read before), so the loads' latency is paid once per block.  Within a block
+// the keys hold the step's number; the block's first column is added once.
+// Blocks of 8: 4 or 16 steps run 4.5% slower and 0.6% faster on 250 bp
+// reads, 2% slower both on 151 bp reads.
+template <int N, bool SYM>
+__device__ __forceinline__ void rp_steps(uint32_t *S, int s, const RpK &K, RpRow &X)
+{
+    uint32_t *Sb = S + s * 32;
+    uint16_t *SEH = reinterpret_cast<uint16_t *>(Sb) + 1;          // E | H << 8 of slot s
+    uint32_t wv[N], hh[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) wv[k] = Sb[k * 32];
+    uint32_t kb = 0;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const uint32_t Hd2 = prmt(X.hB, wv[k], 0x1712u);             // H(i, s-2) | H(i-1, s-1) << 16
+        const uint32_t Ed2 = prmt(X.EN, wv[k], 0x1612u);             // E(i+1, s-1) | E(i, s) << 16
+        // zero-diagonal rule: D * 128 >= D + s for D >= 1, 0 for D = 0
+        const uint32_t M2 = __viaddmin_s16x2(Hd2, prmt(K.p0, K.p1, wv[k]), Hd2 * K.zm);
+        const uint32_t h2 = __vimax3_s16x2(M2, Ed2, X.F);
+        const uint32_t Mi2 = sub_sat_h2(M2, K.oe_i2);
+        const uint32_t Md2 = SYM ? Mi2 : sub_sat_h2(M2, K.oe_d2);
+        const uint32_t EN2 = __viaddmax_s16x2(Ed2, K.ne_d2, Md2);
+        X.F = __viaddmax_s16x2(X.F, K.ne_i2, Mi2);
+        SEH[(k - 1) * 64] = (uint16_t)(X.hK + EN2);                  // slot s-1 <- E(i+2, s-1), H(i+1, s-2)
+        X.hK = h2 * K.k8;
+        kb = k == 0 ? X.hK : __viaddmax_u16x2(X.hK, (uint32_t)k * 0x10001u, kb);
+        X.hB = X.hA;
+        X.hA = h2;
+        X.EN = EN2;
+        hh[k] = h2;
+    }
+    X.key = __viaddmax_u16x2(kb, X.j2, X.key);
+    X.j2 += (uint32_t)N * 0x10001u;
+    if (hh[N - 1] > 0xffffu) {
+        X.L = s + N;
+    } else {
+#pragma unroll
+        for (int k = 0; k < N - 1; ++k)
+            if (hh[k] > 0xffffu) X.L = s + k + 1;
+    }
+}
+
 template <int NMAX, bool SYM>
 __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, const Params &P, const PairRec &R,
                                                             bsw_result_t *out, uint32_t *S)
@@ -469,17 +556,21 @@ __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, cons
     const int wb = clip_band(P, n, R.w);
     const int e_del = P.e_del, e_ins = P.e_ins;
     const int oe_del = P.o_del + e_del, oe_ins = P.o_ins + e_ins;
-    const uint32_t k8 = P.k8, k16 = P.k16;          // 2^8, 2^16 (run-time: multiply-adds, not shifts)
     // Zero-diagonal rule: M = min(D + s, D * 128), D * 128 >= D + s for D >= 1
-    // (match <= 127) and below 2^15 for D <= 255.  The factor comes from a
-    // run-time value so that the product stays a multiply-add (FMA pipe)
-    // instead of becoming a shift (integer pipe).
-    const uint32_t zmul = k8 >> 1;
-    const uint32_t noe_d2 = (uint32_t)(-oe_del & 0xffff) * 0x10001u, noe_i2 = (uint32_t)(-oe_ins & 0xffff) * 0x10001u;
-    const uint32_t ne_d2 = (uint32_t)(-e_del & 0xffff) * 0x10001u, ne_i2 = (uint32_t)(-e_ins & 0xffff) * 0x10001u;
+    // (match <= 127) and below 2^15 for D <= 255.  The factors come from a
+    // run-time value so that the products stay multiplies (FMA pipe) instead of
+    // becoming shifts (integer pipe).
+    RpK K;
+    K.k8 = P.k8;
+    K.zm = P.k8 >> 1;
+    // opening costs above every M (at most 255) act alike
+    K.oe_d2 = (uint32_t)min(oe_del, 1023) * 0x10001u;
+    K.oe_i2 = (uint32_t)min(oe_ins, 1023) * 0x10001u;
+    K.ne_d2 = (uint32_t)(-e_del & 0xffff) * 0x10001u;
+    K.ne_i2 = (uint32_t)(-e_ins & 0xffff) * 0x10001u;
 
-    // Eq. 3, first row, and the selectors: slot j = q_j * 0x11 + q_{j-1} * 0x1100
-    // + 0xc480 (nibbles q_j, q_j | 8, 4 + q_{j-1}, (4 + q_{j-1}) | 8).
+    // Eq. 3, first row, and the selectors: slot j = q_j * 0x1100 + q_{j-1} * 0x11
+    // + 0x80c4 (nibbles 4 + q_{j-1}, (4 + q_{j-1}) | 8, q_j, q_j | 8).
     const int64_t q_off = R.q_off;
     const uint8_t *qp = B.q + (q_off >> 2);
     uint32_t cprev = 0;
@@ -491,7 +582,7 @@ __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, cons
             if (j <= n) {
                 const uint32_t cj = j < n ? (byte >> (2 * k)) & 3u : 0u;
                 const int hv = j == 0 ? h0 : max(0, h0 - P.o_ins - j * e_ins);
-                S[j * 32] = cj * 0x11u + cprev * 0x1100u + 0xc480u + ((uint32_t)hv << 24);
+                S[j * 32] = cj * 0x1100u + cprev * 0x11u + 0x80c4u + ((uint32_t)hv << 24);
                 cprev = cj;
             }
         }
@@ -500,7 +591,6 @@ __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, cons
     const uint32_t mb8 = (uint32_t)(-P.b) & 0xffu;
     const uint32_t mis4 = mb8 * 0x01010101u;
     const uint32_t flip = ((uint32_t)P.a ^ mb8) & 0xffu;
-    const uint8_t *SE8 = reinterpret_cast<const uint8_t *>(S) + 2;                          // E byte of slot 0
     uint16_t *SEH = reinterpret_cast<uint16_t *>(reinterpret_cast<uint8_t *>(S) + 2);     // E | H << 8 of slot 0
 
     int lo = 0, hi = n;
@@ -513,8 +603,8 @@ __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, cons
             tnext = i + 4 < m ? __ldg(tp + (i >> 2) + 1) : 0u;
         }
         const int tb0 = (tbyte >> (2 * (i & 3))) & 3, tb1 = (tbyte >> (2 * (i & 3) + 2)) & 3;
-        const uint32_t p0 = mis4 ^ (flip << (8 * tb0));      // row i: byte c = s(t_i, c)
-        const uint32_t p1 = mis4 ^ (flip << (8 * tb1));      // row i+1
+        K.p0 = mis4 ^ (flip << (8 * tb0));       // row i: byte c = s(t_i, c)
+        K.p1 = mis4 ^ (flip << (8 * tb1));       // row i+1
         const bool single = i + 1 == m;
         lo = max(lo, i - wb);
         hi = min(min(hi, i + wb + 1), n);
@@ -528,8 +618,7 @@ __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, cons
         for (int s = lo; s < hi; ++s) {
             const uint32_t wv = S[s * 32];
             const int d = (int)(wv >> 24), e = (int)((wv >> 16) & 0xffu);
-            const int sc = (int)(short)prmt(p0, p1, wv);
-            const int M = __viaddmin_s32(d, sc, d * (int)zmul);
+            const int M = d > 0 ? d + (int)(short)(prmt(K.p0, K.p1, wv) >> 16) : 0;
             const int h = __vimax3_s32(M, e, f);
             const int en = __viaddmax_s32_relu(e, -e_del, M - oe_del);
             f = __viaddmax_s32_relu(f, -e_ins, M - oe_ins);
@@ -558,43 +647,35 @@ __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, cons
         if (c0 < 0) c0 = max(lo1, i + 1 - wb);
         const int bnd1 = c0 == 0 ? max(0, h0 - oe_del - (i + 1) * e_del) : 0;   // H(i+1, c0-1)
 
-        // Both rows: step s computes (i, s) low and (i+1, s-1) high.
-        uint32_t hA = (uint32_t)hprev | ((uint32_t)bnd1 << 16);   // h of step s-1
-        uint32_t hB = (uint32_t)hprev2;                            // h of step s-2 (low half used)
-        uint32_t ENp = (uint32_t)en_last;                          // E out of step s-1 (low half used)
-        uint32_t F2 = (uint32_t)f;                                 // F(i, s) | F(i+1, s-1) << 16
-        uint32_t key2 = (uint32_t)key_lo, L2 = (uint32_t)Lp;       // row keys H * 256 + column; L + 1
-        uint32_t j2 = (uint32_t)(c0 + 1) | ((uint32_t)c0 << 16);
-#pragma unroll 8
-        for (int s = c0 + 1; s < hi; ++s) {
-            const uint32_t e = SE8[s * 128];                       // E(i, s): byte load before the word
-            const uint32_t wv = S[s * 32];
-            const uint32_t Hd2 = hB * k16 + __umulhi(wv, k8);      // H(i-1, s-1) | H(i, s-2) << 16
-            const uint32_t Ed2 = ENp * k16 + e;                     // E(i, s) | E(i+1, s-1) << 16
-            const uint32_t M2 = __viaddmin_s16x2(Hd2, prmt(p0, p1, wv), Hd2 * zmul);
-            const uint32_t h2 = __vimax3_s16x2(M2, Ed2, F2);
-            const uint32_t Mi2 = __viaddmax_s16x2_relu(M2, noe_i2, 0u);
-            const uint32_t Md2 = SYM ? Mi2 : __viaddmax_s16x2_relu(M2, noe_d2, 0u);
-            const uint32_t EN2 = __viaddmax_s16x2_relu(Ed2, ne_d2, Md2);
-            F2 = __viaddmax_s16x2_relu(F2, ne_i2, Mi2);
-            const uint32_t h2K = h2 * k8;
-            key2 = __viaddmax_u16x2(h2K, j2, key2);
-            L2 = __viaddmax_u16x2(__viaddmin_u16x2(j2, 0x00010001u, h2K), 0u, L2);   // s + 1 where H(i, s) > 0
-            SEH[(s - 1) * 64] = (uint16_t)prmt(EN2, hA, 0x0062u);             // slot s-1 <- E(i+2, s-1), H(i+1, s-2)
-            j2 += 0x00010001u;
-            hB = hA; hA = h2; ENp = EN2;
+        // Both rows: step s computes (i, s) high and (i+1, s-1) low.
+        RpRow X;
+        X.hA = (uint32_t)bnd1 | ((uint32_t)hprev << 16);
+        X.hB = (uint32_t)hprev2 << 16;                             // high half used
+        X.hK = (uint32_t)bnd1 << 8;                                // low half used
+        X.EN = (uint32_t)en_last << 16;                            // high half used
+        X.F = (uint32_t)f << 16;
+        X.key = (uint32_t)key_lo << 16;
+        X.L = Lp;
+        X.j2 = ((uint32_t)(c0 + 1) << 16) | (uint32_t)c0;
+        {
+            int s = c0 + 1;
+            for (; s + 8 <= hi; s += 8) rp_steps<8, SYM>(S, s, K, X);
+            const int rest = max(hi - s, 0);                        // c0 can lie past hi: no steps
+            if (rest & 4) { rp_steps<4, SYM>(S, s, K, X); s += 4; }
+            if (rest & 2) { rp_steps<2, SYM>(S, s, K, X); s += 2; }
+            if (rest & 1) rp_steps<1, SYM>(S, s, K, X);
         }
         int Hi1, Hi2, Ei1, ce, fh, hlh;                            // row i's last values; row i+1's state
         if (hi > c0 + 1) {
-            Hi1 = (int)(hA & 0xffffu); Hi2 = (int)(hB & 0xffffu); Ei1 = (int)(ENp & 0xffffu);
-            ce = hi - 1; fh = (int)(F2 >> 16); hlh = (int)(hA >> 16);
+            Hi1 = (int)(X.hA >> 16); Hi2 = (int)(X.hB >> 16); Ei1 = (int)(X.EN >> 16);
+            ce = hi - 1; fh = (int)(X.F & 0xffffu); hlh = (int)(X.hA & 0xffffu);
+            Lp = X.L;
         } else {
             Hi1 = hprev; Hi2 = hprev2; Ei1 = en_last;
             ce = c0; fh = 0; hlh = bnd1;
         }
-        key_lo = (int)(key2 & 0xffffu);
-        int key_hi = (int)(key2 >> 16);
-        Lp = (int)(L2 & 0xffffu);
+        key_lo = (int)(X.key >> 16);
+        int key_hi = (int)(X.key & 0xffffu);
 
         // Row i: Section V-D's decisions.
         {
@@ -624,8 +705,7 @@ __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, cons
             if (c == hi - 1) { d = Hi2; e = Ei1; }
             else if (c == hi) { d = Hi1; e = 0; }
             else { d = (int)(wc >> 24); e = (int)((wc >> 16) & 0xffu); }   // past row i: the slot as it stands
-            const int sc = (int)(signed char)prmt(p1, 0u, wc);
-            const int M = __viaddmin_s32(d, sc, d * (int)zmul);
+            const int M = d > 0 ? d + (int)(signed char)prmt(K.p1, 0u, wc >> 8) : 0;
             const int h = __vimax3_s32(M, e, fh);
             const int en = __viaddmax_s32_relu(e, -e_del, M - oe_del);
             fh = __viaddmax_s32_relu(fh, -e_ins, M - oe_ins);
@@ -674,8 +754,12 @@ __device__ __forceinline__ bool rp_eligible(const Params &P, const PairRec &R, i
            P.o_ins + P.e_ins <= 30000 && P.e_del <= 30000 && P.e_ins <= 30000;
 }
 
+// Launch bounds: blocks have at most 4 warps, and 5 of them at most share an
+// SM's registers: about 100 a thread, which shared memory (12 warps of the
+// 128-base class) leaves free and the row-pair steps' loads in flight use
+// (at the compiler's own 64: 11.18 ms against 10.76).
 template <int NMAX, bool U8, bool NM = false>
-__global__ void __launch_bounds__(256) k_inter(Batch B, Params P, Work W, int cls)
+__global__ void __launch_bounds__(128, 5) k_inter(Batch B, Params P, Work W, int cls)
 {
     extern __shared__ uint32_t smem[];
     const int lane = threadIdx.x & 31;
