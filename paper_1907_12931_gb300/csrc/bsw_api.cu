@@ -245,7 +245,7 @@ struct Lane {
     int create()
     {
         if (cudaStreamCreateWithFlags(&S.main, cudaStreamNonBlocking) != cudaSuccess) return BSW_ECUDA;
-        for (int k = 0; k < 3; ++k) {
+        for (int k = 0; k < kSideStreams; ++k) {
             if (cudaStreamCreateWithFlags(&S.side[k], cudaStreamNonBlocking) != cudaSuccess) return BSW_ECUDA;
             if (cudaEventCreateWithFlags(&S.join[k], cudaEventDisableTiming) != cudaSuccess) return BSW_ECUDA;
         }
@@ -257,7 +257,7 @@ struct Lane {
     void destroy(Budget &B)
     {
         if (S.main) cudaStreamSynchronize(S.main);
-        for (int k = 0; k < 3; ++k) {
+        for (int k = 0; k < kSideStreams; ++k) {
             if (S.side[k]) { cudaStreamSynchronize(S.side[k]); cudaStreamDestroy(S.side[k]); }
             if (S.join[k]) cudaEventDestroy(S.join[k]);
         }

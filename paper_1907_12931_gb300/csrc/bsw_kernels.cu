@@ -2211,10 +2211,20 @@ constexpr ClassLaunch kClassLaunch[kNumClass + 1] = {
     cls_i16<256>, cls_i16<128>, cls_i16<64>, cls_i16<32>, cls_cta, cls_w16, cls_w32, cls_w32};
 
 // Launch order of the classes in the forked path and the side stream of each:
-// the longest work first (block-per-pair pairs, then the long 8-bit
-// classes), each stream ending with shorter work.
+// the longest work first (block-per-pair pairs, then the long 8-bit classes).
+// A class with few pairs lasts as long as its longest warp, 50 to 300 us
+// whatever its size, so in a small batch classes that usually hold pairs
+// together share no stream (10 k short pairs: 416 us, against 1010 with three
+// streams; 400 k pairs of 151 bp reads: 643 against 801 with four).  A large
+// batch fills the SMs with one class at a time and loses when all of them are
+// resident in turns, so pairs of neighbouring classes share a stream (2 M pairs
+// of 151 bp reads: 2.27 ms against 2.46 with eight streams; 1 M pairs of 250 bp
+// reads with N: 4.52 against 5.06).  The line lies between 250 bp reads, where
+// the two meet near 350 k pairs, and 151 bp reads, where they do near 550 k.
+constexpr int64_t kSpreadPairs = 393216;
 constexpr int kForkOrder[kNumClass] = {kClsCTA, 0, 1, 2, 3, 4, 5, 6, 7, kClsW16, kClsW32, 8, 9, 10, 11};
-constexpr int kClassStream[kNumClass] = {0, 0, 0, 1, 1, 1, 2, 2, 2, 2, 2, 2, 0, 2, 2};
+constexpr int kClassStreamSmall[kNumClass] = {0, 1, 2, 3, 4, 5, 6, 7, 0, 1, 2, 3, 3, 5, 6};
+constexpr int kClassStreamLarge[kNumClass] = {0, 0, 1, 1, 2, 2, 3, 3, 0, 1, 2, 3, 3, 2, 2};
 
 // Whether class c can hold pairs under the plan and the batch flags (classes
 // that cannot are not launched).
@@ -2337,9 +2347,10 @@ cudaError_t launch_batched(const Batch &B, const Params &P0, const Work &W, cons
     // Fork: classes run concurrently on the side streams so that one class's
     // tail overlaps the next class's start.
     if ((e = cudaEventRecord(S.fork, S.main)) != cudaSuccess) return e;
-    for (int k = 0; k < 3; ++k)
+    for (int k = 0; k < kSideStreams; ++k)
         if ((e = cudaStreamWaitEvent(S.side[k], S.fork, 0)) != cudaSuccess) return e;
     const int wblocks = sms * kWarpBlocksPerSM;
+    const int *side = B.n <= kSpreadPairs ? kClassStreamSmall : kClassStreamLarge;
     // The two-columns warp kernel runs after the other classes: it leaves a
     // quarter of each SM's block slots free (3 blocks of its 4, so the
     // longest pairs get a twelfth of an SM, not a sixteenth), and kernels of
@@ -2347,9 +2358,9 @@ cudaError_t launch_batched(const Batch &B, const Params &P0, const Work &W, cons
     const bool x2_after = L.warp_x2 && x2_usable(P) && x2_ring_log2(P) > 0;
     for (int c : kForkOrder)
         if (class_live(c, L, P.flags) && !(x2_after && c == kClsW16) &&
-            (e = launch_class(c, B, P, W, S.side[kClassStream[c]], sms, wblocks, L, T)) != cudaSuccess)
+            (e = launch_class(c, B, P, W, S.side[side[c]], sms, wblocks, L, T)) != cudaSuccess)
             return e;
-    for (int k = 0; k < 3; ++k) {
+    for (int k = 0; k < kSideStreams; ++k) {
         if ((e = cudaEventRecord(S.join[k], S.side[k])) != cudaSuccess) return e;
         if ((e = cudaStreamWaitEvent(S.main, S.join[k], 0)) != cudaSuccess) return e;
     }

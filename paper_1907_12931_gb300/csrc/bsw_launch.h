@@ -19,11 +19,15 @@ constexpr int kWarpBlocksPerSM = 2;
 constexpr int kU8Nmax[8] = {256, 224, 192, 160, 128, 96, 64, 32};
 constexpr int kI16Nmax[4] = {256, 128, 64, 32};
 
+// Side streams the class kernels fork over: as many as there are 8-bit
+// classes, so that in small batches no two of them wait for each other.
+constexpr int kSideStreams = 8;
+
 struct Streams {
     cudaStream_t main;
-    cudaStream_t side[3];
+    cudaStream_t side[kSideStreams];
     cudaEvent_t fork;
-    cudaEvent_t join[3];
+    cudaEvent_t join[kSideStreams];
 };
 
 // How one batch is laid out over the kernels: which query lengths run one
