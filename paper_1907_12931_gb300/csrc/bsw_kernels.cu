@@ -436,16 +436,16 @@ __device__ __forceinline__ unsigned long long inter_pair(const Batch &B, const P
 
 // ------------------------------------------ two rows per instruction (8-bit)
 //
-// The 8-bit class pairs without N bases take rows in pairs: rows i and i+1 sit
+// The 8-bit class pairs take rows in pairs: rows i and i+1 sit
 // in the high and low halves of s16x2 registers, row i+1 one column behind
 // (step s computes cells (i, s) and (i+1, s-1)), so every DPX instruction of
 // the cell update (Eq. 2, Eq. 3's affine gaps) advances two cells.  Row i+1
 // takes its diagonal H(i, s-2) and its E(i+1, s-1) from row i's registers;
 // only row i+1's results go back to the slot column, slot s-1 <- {H(i+1, s-2),
 // E(i+2, s-1)}, so a pass reads each slot once and writes it once for two
-// rows.  The row selector in bits 0-15 of slot s picks byte q_s of row i's
-// profile for the high half and byte 4 + q_{s-1} (row i+1's profile) for the
-// low half, both sign-extended, so one byte permute gives both scores.
+// rows.  The row selector in bits 0-15 of slot s picks byte 4 + q_s (row i's
+// profile) for the high half and byte q_{s-1} of row i+1's profile for the low
+// half, both sign-extended, so one byte permute gives both scores.
 //
 // Row i+1's band depends on row i's rule-c trims, which are known only after
 // row i ends.  Its left end is found before the packed loop starts: row i
@@ -487,6 +487,8 @@ __device__ __forceinline__ uint32_t sub_sat_h2(uint32_t a, uint32_t b)
     return d;
 }
 
+constexpr uint32_t kNScore = 0xffffffffu;   // an N scores -1 against anything
+
 // A thread's constants and running values of the row-pair pass: high halves
 // row i, low halves row i + 1.
 struct RpK {
@@ -503,13 +505,25 @@ struct RpRow {
     int L;                                  // last column of row i with H > 0, plus 1
 };
 
+// Scores of the selectors in a slot word: row i's high, row i+1's low.  Without
+// N one permute over both profiles gives them.  With N in the queries (NM) a
+// selector's nibbles run over five codes, byte 4 being N's -1, so each profile
+// takes a permute of its own and a third joins the halves (1 M pairs of 250 bp
+// reads with 0.1% N: 3.15 ms, 2.8 without N, 4.54 with one row per pass).
+template <bool NM>
+__device__ __forceinline__ uint32_t rp_scores(const RpK &K, uint32_t wv)
+{
+    if (!NM) return prmt(K.p1, K.p0, wv);
+    return prmt(prmt(K.p1, kNScore, wv), prmt(K.p0, kNScore, wv), 0x7610u);
+}
+
 // N steps from step s: cells (i, s + k) and (i + 1, s + k - 1).  All N slots
 // are read before the first is written back (step s + k writes slot s + k - 1,
 // read before), so the loads' latency is paid once per block.  Within a block
 // the keys hold the step's number; the block's first column is added once.
 // Blocks of 8: 4 or 16 steps run 4.5% slower and 0.6% faster on 250 bp
 // reads, 2% slower both on 151 bp reads.
-template <int N, bool SYM>
+template <int N, bool SYM, bool NM>
 __device__ __forceinline__ void rp_steps(uint32_t *S, int s, const RpK &K, RpRow &X)
 {
     uint32_t *Sb = S + s * 32;
@@ -523,7 +537,7 @@ __device__ __forceinline__ void rp_steps(uint32_t *S, int s, const RpK &K, RpRow
         const uint32_t Hd2 = prmt(X.hB, wv[k], 0x1712u);             // H(i, s-2) | H(i-1, s-1) << 16
         const uint32_t Ed2 = prmt(X.EN, wv[k], 0x1612u);             // E(i+1, s-1) | E(i, s) << 16
         // zero-diagonal rule: D * 128 >= D + s for D >= 1, 0 for D = 0
-        const uint32_t M2 = __viaddmin_s16x2(Hd2, prmt(K.p0, K.p1, wv[k]), Hd2 * K.zm);
+        const uint32_t M2 = __viaddmin_s16x2(Hd2, rp_scores<NM>(K, wv[k]), Hd2 * K.zm);
         const uint32_t h2 = __vimax3_s16x2(M2, Ed2, X.F);
         const uint32_t Mi2 = sub_sat_h2(M2, K.oe_i2);
         const uint32_t Md2 = SYM ? Mi2 : sub_sat_h2(M2, K.oe_d2);
@@ -548,7 +562,7 @@ __device__ __forceinline__ void rp_steps(uint32_t *S, int s, const RpK &K, RpRow
     }
 }
 
-template <int NMAX, bool SYM>
+template <bool SYM, bool NM>
 __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, const Params &P, const PairRec &R,
                                                             bsw_result_t *out, uint32_t *S)
 {
@@ -570,24 +584,35 @@ __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, cons
     K.ne_i2 = (uint32_t)(-e_ins & 0xffff) * 0x10001u;
 
     // Eq. 3, first row, and the selectors: slot j = q_j * 0x1100 + q_{j-1} * 0x11
-    // + 0x80c4 (nibbles 4 + q_{j-1}, (4 + q_{j-1}) | 8, q_j, q_j | 8).
+    // + 0x8480 (nibbles q_{j-1}, q_{j-1} | 8, 4 + q_j, (4 + q_j) | 8), or without
+    // the 4's with N codes.
+    constexpr uint32_t kSel = NM ? 0x8080u : 0xc480u;
     const int64_t q_off = R.q_off;
     const uint8_t *qp = B.q + (q_off >> 2);
     uint32_t cprev = 0;
     for (int c = 0; c <= n; c += 4) {
         const uint32_t byte = c < n ? __ldg(qp + (c >> 2)) : 0u;
+        const uint32_t nb = (NM && B.q_n && c < n) ? (uint32_t)__ldg(B.q_n + ((q_off + c) >> 3)) >> ((q_off + c) & 7) : 0u;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int j = c + k;
             if (j <= n) {
-                const uint32_t cj = j < n ? (byte >> (2 * k)) & 3u : 0u;
+                const uint32_t cj = j >= n ? 0u : NM && ((nb >> k) & 1u) ? 4u : (byte >> (2 * k)) & 3u;
                 const int hv = j == 0 ? h0 : max(0, h0 - P.o_ins - j * e_ins);
-                S[j * 32] = cj * 0x1100u + cprev * 0x11u + 0x80c4u + ((uint32_t)hv << 24);
+                S[j * 32] = cj * 0x1100u + cprev * 0x11u + kSel + ((uint32_t)hv << 24);
                 cprev = cj;
             }
         }
     }
-    const uint8_t *tp = B.t + (R.t_off >> 2);
+    const uint8_t *tn = NM ? B.t_n : nullptr;
+    const int64_t t_off = R.t_off;
+    const uint8_t *tp = B.t + (t_off >> 2);
+    // four rows' bases and, in bits 8-11, their N bits
+    auto t_rows = [&](int i) {
+        uint32_t v = __ldg(tp + (i >> 2));
+        if (NM && tn) v |= (((uint32_t)__ldg(tn + ((t_off + i) >> 3)) >> ((t_off + i) & 7)) & 15u) << 8;
+        return v;
+    };
     const uint32_t mb8 = (uint32_t)(-P.b) & 0xffu;
     const uint32_t mis4 = mb8 * 0x01010101u;
     const uint32_t flip = ((uint32_t)P.a ^ mb8) & 0xffu;
@@ -596,15 +621,17 @@ __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, cons
     int lo = 0, hi = n;
     int best = h0, bi = -1, bj = -1, gbest = -1, gi = -1, moff = 0;
     unsigned long long ncell = 0;
-    uint32_t tbyte = 0, tnext = __ldg(tp);                  // target bases, fetched one byte (4 rows) ahead
+    uint32_t tbyte = 0, tnext = t_rows(0);                  // target bases, fetched one byte (4 rows) ahead
     for (int i = 0; i < m; i += 2) {
         if ((i & 3) == 0) {
             tbyte = tnext;
-            tnext = i + 4 < m ? __ldg(tp + (i >> 2) + 1) : 0u;
+            tnext = i + 4 < m ? t_rows(i + 4) : 0u;
         }
         const int tb0 = (tbyte >> (2 * (i & 3))) & 3, tb1 = (tbyte >> (2 * (i & 3) + 2)) & 3;
         K.p0 = mis4 ^ (flip << (8 * tb0));       // row i: byte c = s(t_i, c)
         K.p1 = mis4 ^ (flip << (8 * tb1));       // row i+1
+        if (NM && ((tbyte >> (8 + (i & 3))) & 1u)) K.p0 = kNScore;
+        if (NM && ((tbyte >> (9 + (i & 3))) & 1u)) K.p1 = kNScore;
         const bool single = i + 1 == m;
         lo = max(lo, i - wb);
         hi = min(min(hi, i + wb + 1), n);
@@ -618,7 +645,7 @@ __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, cons
         for (int s = lo; s < hi; ++s) {
             const uint32_t wv = S[s * 32];
             const int d = (int)(wv >> 24), e = (int)((wv >> 16) & 0xffu);
-            const int M = d > 0 ? d + (int)(short)(prmt(K.p0, K.p1, wv) >> 16) : 0;
+            const int M = d > 0 ? d + ((int)rp_scores<NM>(K, wv) >> 16) : 0;
             const int h = __vimax3_s32(M, e, f);
             const int en = __viaddmax_s32_relu(e, -e_del, M - oe_del);
             f = __viaddmax_s32_relu(f, -e_ins, M - oe_ins);
@@ -659,11 +686,11 @@ __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, cons
         X.j2 = ((uint32_t)(c0 + 1) << 16) | (uint32_t)c0;
         {
             int s = c0 + 1;
-            for (; s + 8 <= hi; s += 8) rp_steps<8, SYM>(S, s, K, X);
+            for (; s + 8 <= hi; s += 8) rp_steps<8, SYM, NM>(S, s, K, X);
             const int rest = max(hi - s, 0);                        // c0 can lie past hi: no steps
-            if (rest & 4) { rp_steps<4, SYM>(S, s, K, X); s += 4; }
-            if (rest & 2) { rp_steps<2, SYM>(S, s, K, X); s += 2; }
-            if (rest & 1) rp_steps<1, SYM>(S, s, K, X);
+            if (rest & 4) { rp_steps<4, SYM, NM>(S, s, K, X); s += 4; }
+            if (rest & 2) { rp_steps<2, SYM, NM>(S, s, K, X); s += 2; }
+            if (rest & 1) rp_steps<1, SYM, NM>(S, s, K, X);
         }
         int Hi1, Hi2, Ei1, ce, fh, hlh;                            // row i's last values; row i+1's state
         if (hi > c0 + 1) {
@@ -705,7 +732,7 @@ __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, cons
             if (c == hi - 1) { d = Hi2; e = Ei1; }
             else if (c == hi) { d = Hi1; e = 0; }
             else { d = (int)(wc >> 24); e = (int)((wc >> 16) & 0xffu); }   // past row i: the slot as it stands
-            const int M = d > 0 ? d + (int)(signed char)prmt(K.p1, 0u, wc >> 8) : 0;
+            const int M = d > 0 ? d + (int)(signed char)prmt(K.p1, kNScore, (wc >> 8) & (NM ? 7u : 3u)) : 0;
             const int h = __vimax3_s32(M, e, fh);
             const int en = __viaddmax_s32_relu(e, -e_del, M - oe_del);
             fh = __viaddmax_s32_relu(fh, -e_ins, M - oe_ins);
@@ -744,21 +771,59 @@ __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, cons
     return ncell;
 }
 
-// Whether the row-pair path takes the pair: no N bases (the caller's kernel
-// runs it only for batches without N bitmaps), scores and gap terms inside
-// the packed 8-bit range.
-__device__ __forceinline__ bool rp_eligible(const Params &P, const PairRec &R, int nmax)
+// The next group of 32 pairs of class cls for a warp, or -1.
+__device__ __forceinline__ int next_group(const Work &W, int cls, int lane, int ngroups)
 {
-    return R.n >= 1 && R.m >= 1 && R.n <= nmax && R.h0 >= 0 &&
-           (long long)R.h0 + (long long)P.a * min(R.n, R.m) <= 255 && P.a <= 127 && P.o_del + P.e_del <= 30000 &&
-           P.o_ins + P.e_ins <= 30000 && P.e_del <= 30000 && P.e_ins <= 30000;
+    int g = 0;
+    if (lane == 0) g = (int)atomicAdd(&W.cls_next[cls], 1u);
+    g = __shfl_sync(kFull, g, 0);
+    return g < ngroups ? g : -1;
 }
 
-// Launch bounds: blocks have at most 4 warps, and 5 of them at most share an
-// SM's registers: about 100 a thread, which shared memory (12 warps of the
-// 128-base class) leaves free and the row-pair steps' loads in flight use
-// (at the compiler's own 64: 11.18 ms against 10.76).
-template <int NMAX, bool U8, bool NM = false>
+// Fields of entry idx of the sorted order (pair p).
+__device__ __forceinline__ PairRec pair_rec(const Batch &B, const Params &P, const Work &W, int idx, int p)
+{
+    if (W.rec) return W.rec[idx];
+    PairRec R;
+    R.q_off = B.q_off[p]; R.t_off = B.t_off[p];
+    R.n = B.q_len[p]; R.m = B.t_len[p]; R.h0 = B.h0[p];
+    R.w = B.w_override ? B.w_override[p] : P.w;
+    return R;
+}
+
+// Persistent kernel of an 8-bit class with two rows per instruction: warps
+// take groups of 32 pairs of the sorted order, one pair per lane, with nmax + 1
+// slots of shared memory each (nmax the class's bound).  NM: the batch has N
+// bitmaps.
+// Launch bounds: blocks have at most 4 warps, and 6 of them at most share an
+// SM's registers: up to 85 a thread, which the steps' loads in flight use (4 M
+// pairs of 250 bp reads: 10.85 ms; 5 blocks 11.04, 4 blocks 11.19, 64 registers
+// 11.18; shared memory holds 12 warps of the 128-base class).  With N bases the
+// two more permutes a step want 5 (1 M pairs: 3.15 ms against 3.25).
+template <bool SYM, bool NM>
+__global__ void __launch_bounds__(128, NM ? 5 : 6) k_rows2(Batch B, Params P, Work W, int cls, int nmax)
+{
+    extern __shared__ uint32_t smem[];
+    const int lane = threadIdx.x & 31;
+    uint32_t *S = smem + (threadIdx.x >> 5) * ((nmax + 1) * 32) + lane;
+    const int start = W.cls_start[cls], count = W.cls_count[cls];
+    const int ngroups = (count + 31) >> 5;
+    unsigned long long cells = 0;
+    for (int g; (g = next_group(W, cls, lane, ngroups)) >= 0;) {
+        const int idx = (g << 5) + lane;
+        if (idx < count) {
+            const int p = W.order[start + idx];
+            cells += inter_pair_rp<SYM, NM>(B, P, pair_rec(B, P, W, start + idx, p), &B.out[p], S);
+        }
+        __syncwarp();
+    }
+    for (int d = 16; d > 0; d >>= 1) cells += __shfl_xor_sync(kFull, cells, d);
+    if (lane == 0 && cells) atomicAdd(W.cells, cells);
+}
+
+// Persistent kernel with one row at a time: the 16-bit classes, and the 8-bit
+// ones where k_rows2 does not apply (rows2_ok), which take batches with N too.
+template <int NMAX, bool U8>
 __global__ void __launch_bounds__(128, 5) k_inter(Batch B, Params P, Work W, int cls)
 {
     extern __shared__ uint32_t smem[];
@@ -767,28 +832,11 @@ __global__ void __launch_bounds__(128, 5) k_inter(Batch B, Params P, Work W, int
     const int start = W.cls_start[cls], count = W.cls_count[cls];
     const int ngroups = (count + 31) >> 5;
     unsigned long long cells = 0;
-    for (;;) {
-        int g = 0;
-        if (lane == 0) g = (int)atomicAdd(&W.cls_next[cls], 1u);
-        g = __shfl_sync(kFull, g, 0);
-        if (g >= ngroups) break;
+    for (int g; (g = next_group(W, cls, lane, ngroups)) >= 0;) {
         const int idx = (g << 5) + lane;
         if (idx < count) {
             const int p = W.order[start + idx];
-            PairRec R;
-            if (W.rec) {
-                R = W.rec[start + idx];
-            } else {
-                R.q_off = B.q_off[p]; R.t_off = B.t_off[p];
-                R.n = B.q_len[p]; R.m = B.t_len[p]; R.h0 = B.h0[p];
-                R.w = B.w_override ? B.w_override[p] : P.w;
-            }
-            if (U8 && !NM && rp_eligible(P, R, NMAX)) {
-                cells += (P.o_del == P.o_ins && P.e_del == P.e_ins) ? inter_pair_rp<NMAX, true>(B, P, R, &B.out[p], S)
-                                                                   : inter_pair_rp<NMAX, false>(B, P, R, &B.out[p], S);
-            } else {
-                cells += inter_pair<NMAX, U8, NM>(B, P, W, p, R, S);
-            }
+            cells += inter_pair<NMAX, U8, U8>(B, P, W, p, pair_rec(B, P, W, start + idx, p), S);
         }
         __syncwarp();
     }
@@ -2026,14 +2074,15 @@ Plan default_plan()
 
 namespace {
 
-// Resident blocks per SM of each k_inter instantiation with 1, 2 and 4 warps
-// per block, set by prepare_kernels.
-int g_inter_blocks[12][3];
-int g_inter_blocks_n[8][3];     // the N-aware 8-bit instantiations
+// Resident blocks per SM of each per-thread class's kernels with 1, 2 and 4
+// warps per block, set by prepare_kernels.
+int g_inter_blocks[12][3];      // k_inter
+int g_rows2_blocks[2][8][3];    // k_rows2, without and with N
 
 int warps_index(int warps) { return warps <= 1 ? 0 : warps == 2 ? 1 : 2; }
 
-template <int NMAX, bool U8> size_t inter_smem(int warps) { return (size_t)warps * (NMAX + 1) * 32 * 4; }
+// A slot column of 32-bit words per lane, for either per-thread kernel.
+size_t inter_smem(int nmax, int warps) { return (size_t)warps * (nmax + 1) * 32 * 4; }
 template <int NMAX, bool U8> constexpr int inter_index()
 {
     return U8 ? (NMAX >= 256 ? 0 : NMAX >= 224 ? 1 : NMAX >= 192 ? 2 : NMAX >= 160 ? 3 : NMAX >= 128 ? 4 : NMAX >= 96 ? 5
@@ -2041,40 +2090,54 @@ template <int NMAX, bool U8> constexpr int inter_index()
               : 8 + (NMAX >= 256 ? 0 : NMAX >= 128 ? 1 : NMAX >= 64 ? 2 : 3);
 }
 
-template <int NMAX, bool U8, bool NM>
-cudaError_t prepare_inter_one(int *blocks)
+// The kernel's shared-memory limit, and its resident blocks with queries up
+// to nmax bases.
+template <class K>
+cudaError_t prepare_slots(K *kernel, int nmax, int *blocks)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_inter<NMAX, U8, NM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)inter_smem<NMAX, U8>(4));
-    if (e != cudaSuccess) return e;
-    for (int wi = 0; wi < 3; ++wi) {
-        const int warps = 1 << wi;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)inter_smem(kShortMax, 4));
+    for (int wi = 0; wi < 3 && e == cudaSuccess; ++wi) {
         int nb = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_inter<NMAX, U8, NM>, warps * 32,
-                                                          inter_smem<NMAX, U8>(warps));
-        if (e != cudaSuccess) return e;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, 32 << wi, inter_smem(nmax, 1 << wi));
         blocks[wi] = nb > 0 ? nb : 1;
     }
-    return cudaSuccess;
+    return e;
 }
 
+// The 8-bit instantiations of k_inter are the N-aware ones (they take batches
+// without N too); split gap costs need no more of an SM than equal ones.
 template <int NMAX, bool U8>
 cudaError_t prepare_inter()
 {
-    cudaError_t e = prepare_inter_one<NMAX, U8, false>(g_inter_blocks[inter_index<NMAX, U8>()]);
+    constexpr int c = inter_index<NMAX, U8>();
+    cudaError_t e = prepare_slots(k_inter<NMAX, U8>, NMAX, g_inter_blocks[c]);
     if (e != cudaSuccess || !U8) return e;
-    return prepare_inter_one<NMAX, true, true>(g_inter_blocks_n[inter_index<NMAX, U8>()]);
+    int unused[3];
+    if ((e = prepare_slots(k_rows2<false, false>, NMAX, unused)) != cudaSuccess) return e;
+    if ((e = prepare_slots(k_rows2<false, true>, NMAX, unused)) != cudaSuccess) return e;
+    if ((e = prepare_slots(k_rows2<true, false>, NMAX, g_rows2_blocks[0][c & 7])) != cudaSuccess) return e;
+    return prepare_slots(k_rows2<true, true>, NMAX, g_rows2_blocks[1][c & 7]);
+}
+
+// Whether the 8-bit classes run two rows per instruction: the gap costs fit
+// the packed halves and the score bound was checked (lanes not forced).
+bool rows2_ok(const Params &P)
+{
+    return !(P.flags & BSW_FORCE_I8) && P.o_del + P.e_del <= 30000 && P.o_ins + P.e_ins <= 30000;
 }
 
 template <int NMAX, bool U8>
 cudaError_t launch_inter(const Batch &B, const Params &P, const Work &W, int cls, cudaStream_t st, int sms, int warps)
 {
-    if (U8 && (B.q_n || B.t_n)) {
-        const int blocks = sms * g_inter_blocks_n[inter_index<NMAX, U8>()][warps_index(warps)];
-        k_inter<NMAX, true, true><<<blocks, warps * 32, inter_smem<NMAX, U8>(warps), st>>>(B, P, W, cls);
+    constexpr int c = inter_index<NMAX, U8>();
+    const size_t smem = inter_smem(NMAX, warps);
+    if (U8 && rows2_ok(P)) {
+        const bool nm = B.q_n || B.t_n, sym = P.o_del == P.o_ins && P.e_del == P.e_ins;
+        const int blocks = sms * g_rows2_blocks[nm][c & 7][warps_index(warps)];
+        auto *k = nm ? (sym ? k_rows2<true, true> : k_rows2<false, true>) : (sym ? k_rows2<true, false> : k_rows2<false, false>);
+        k<<<blocks, warps * 32, smem, st>>>(B, P, W, cls, NMAX);
     } else {
-        const int blocks = sms * g_inter_blocks[inter_index<NMAX, U8>()][warps_index(warps)];
-        k_inter<NMAX, U8, false><<<blocks, warps * 32, inter_smem<NMAX, U8>(warps), st>>>(B, P, W, cls);
+        k_inter<NMAX, U8><<<sms * g_inter_blocks[c][warps_index(warps)], warps * 32, smem, st>>>(B, P, W, cls);
     }
     return cudaGetLastError();
 }
