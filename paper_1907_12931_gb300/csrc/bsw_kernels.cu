@@ -11,9 +11,12 @@
 // Kernels
 //   k_classify/k_scan/k_scatter  length bucketing (Section V-C1's sort by
 //                                length, as a device counting sort)
-//   k_inter<NMAX, U8>            one pair per thread: the paper's inter-task
-//                                SIMD (Section V-C) mapped onto SIMT lanes;
-//                                8-bit or 16-bit lanes (Section V-D1)
+//   k_rows2, k_rows2_16          one pair per thread: the paper's inter-task
+//                                SIMD (Section V-C) mapped onto SIMT lanes,
+//                                two rows of the pair per packed instruction;
+//                                8-bit and 16-bit lanes (Section V-D1)
+//   k_rows1                      the same with one row at a time: forced 8-bit
+//                                lanes and gap costs past 16 bits
 //   k_warp<C, S16>               one pair per warp, row-synchronous: each lane
 //                                owns C consecutive columns of a row chunk and
 //                                F is a max-plus scan across lanes; used for
@@ -290,16 +293,16 @@ __device__ __forceinline__ bool slot_nonzero(uint32_t w)
 // re-run when a score leaves the lane range.
 // NM: the batch has N bitmaps (8-bit lanes only); kernels of batches without
 // them carry no N code.
-template <int NMAX, bool U8, bool NM>
+template <bool U8, bool NM>
 __device__ __forceinline__ unsigned long long inter_pair(const Batch &B, const Params &P, const Work &W,
-                                                         int p, const PairRec &R, uint32_t *S)
+                                                         int p, const PairRec &R, uint32_t *S, int nmax)
 {
     constexpr int VMAX = U8 ? 255 : 32767;
     const int n = R.n, m = R.m, h0 = R.h0;
     const int wb = clip_band(P, n, R.w);
     const int e_del = P.e_del, e_ins = P.e_ins;
     const int oe_del = P.o_del + e_del, oe_ins = P.o_ins + e_ins;
-    if (h0 > VMAX || n > NMAX) {
+    if (h0 > VMAX || n > nmax) {
         W.rerun[atomicAdd(&W.cls_count[kRerun], 1)] = p;
         return 0;
     }
@@ -487,123 +490,297 @@ __device__ __forceinline__ uint32_t sub_sat_h2(uint32_t a, uint32_t b)
     return d;
 }
 
+// Per half of a non-negative number below 31744: 15360 (1.0's bits) if it is
+// positive, 0 if it is 0.  x * infinity is infinity, which .sat makes 1.0, or
+// for x = 0 a NaN, which it makes +0.
+__device__ __forceinline__ uint32_t positive_h2(uint32_t x)
+{
+    uint32_t d;
+    asm("mul.rn.sat.f16x2 %0, %1, %2;" : "=r"(d) : "r"(x), "r"(0x7c007c00u));
+    return d;
+}
+
 constexpr uint32_t kNScore = 0xffffffffu;   // an N scores -1 against anything
 
-// A thread's constants and running values of the row-pair pass: high halves
-// row i, low halves row i + 1.
-struct RpK {
-    uint32_t p0, p1;                        // byte c: score of (t_i, c), (t_{i+1}, c)
-    uint32_t oe_d2, oe_i2, ne_d2, ne_i2;    // o + e; -e
-    uint32_t k8, zm;                        // 2^8 and the zero-diagonal factor 2^7
-};
+// Running values of a row-pair pass: high halves row i, low halves row i + 1.
 struct RpRow {
     uint32_t hA, hB;                        // H of steps s - 1 and s - 2
-    uint32_t hK;                            // hA * 256
+    uint32_t hK;                            // hA * 256 (8-bit lanes)
     uint32_t EN, F;                         // E out of step s - 1; F into step s
-    uint32_t key;                           // row keys H * 256 + column
-    uint32_t j2;                            // s << 16 | s - 1
+    uint32_t key, j2;                       // 8-bit lanes: row keys H * 256 + column; s << 16 | s - 1
+    int k0, k1;                             // 16-bit lanes: row keys H * 512 + column of rows i, i + 1
     int L;                                  // last column of row i with H > 0, plus 1
+
+    // The last column of row i with H > 0 once steps s..s+N-1 have given hh.
+    template <int N>
+    __device__ __forceinline__ void settle(int s, const uint32_t (&hh)[N])
+    {
+        if (hh[N - 1] > 0xffffu) {
+            L = s + N;
+        } else {
+#pragma unroll
+            for (int k = 0; k < N - 1; ++k)
+                if (hh[k] > 0xffffu) L = s + k + 1;
+        }
+    }
 };
 
-// Scores of the selectors in a slot word: row i's high, row i+1's low.  Without
-// N one permute over both profiles gives them.  With N in the queries (NM) a
-// selector's nibbles run over five codes, byte 4 being N's -1, so each profile
-// takes a permute of its own and a third joins the halves (1 M pairs of 250 bp
-// reads with 0.1% N: 3.15 ms, 2.8 without N, 4.54 with one row per pass).
-template <bool NM>
-__device__ __forceinline__ uint32_t rp_scores(const RpK &K, uint32_t wv)
-{
-    if (!NM) return prmt(K.p1, K.p0, wv);
-    return prmt(prmt(K.p1, kNScore, wv), prmt(K.p0, kNScore, wv), 0x7610u);
-}
+// The constants of a lane's cells: scores of its two rows by query code (byte
+// c: score of base c), o + e and -e in both halves.
+struct RpK {
+    uint32_t p0, p1, oe_d2, oe_i2, ne_d2, ne_i2;
 
-// N steps from step s: cells (i, s + k) and (i + 1, s + k - 1).  All N slots
-// are read before the first is written back (step s + k writes slot s + k - 1,
-// read before), so the loads' latency is paid once per block.  Within a block
-// the keys hold the step's number; the block's first column is added once.
-// Blocks of 8: 4 or 16 steps run 4.5% slower and 0.6% faster on 250 bp
-// reads, 2% slower both on 151 bp reads.
-template <int N, bool SYM, bool NM>
-__device__ __forceinline__ void rp_steps(uint32_t *S, int s, const RpK &K, RpRow &X)
-{
-    uint32_t *Sb = S + s * 32;
-    uint16_t *SEH = reinterpret_cast<uint16_t *>(Sb) + 1;          // E | H << 8 of slot s
-    uint32_t wv[N], hh[N];
-#pragma unroll
-    for (int k = 0; k < N; ++k) wv[k] = Sb[k * 32];
-    uint32_t kb = 0;
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-        const uint32_t Hd2 = prmt(X.hB, wv[k], 0x1712u);             // H(i, s-2) | H(i-1, s-1) << 16
-        const uint32_t Ed2 = prmt(X.EN, wv[k], 0x1612u);             // E(i+1, s-1) | E(i, s) << 16
-        // zero-diagonal rule: D * 128 >= D + s for D >= 1, 0 for D = 0
-        const uint32_t M2 = __viaddmin_s16x2(Hd2, rp_scores<NM>(K, wv[k]), Hd2 * K.zm);
-        const uint32_t h2 = __vimax3_s16x2(M2, Ed2, X.F);
-        const uint32_t Mi2 = sub_sat_h2(M2, K.oe_i2);
-        const uint32_t Md2 = SYM ? Mi2 : sub_sat_h2(M2, K.oe_d2);
-        const uint32_t EN2 = __viaddmax_s16x2(Ed2, K.ne_d2, Md2);
-        X.F = __viaddmax_s16x2(X.F, K.ne_i2, Mi2);
-        SEH[(k - 1) * 64] = (uint16_t)(X.hK + EN2);                  // slot s-1 <- E(i+2, s-1), H(i+1, s-2)
-        X.hK = h2 * K.k8;
-        kb = k == 0 ? X.hK : __viaddmax_u16x2(X.hK, (uint32_t)k * 0x10001u, kb);
-        X.hB = X.hA;
-        X.hA = h2;
-        X.EN = EN2;
-        hh[k] = h2;
+    // top: an opening cost above every M acts like any larger one
+    __device__ __forceinline__ RpK(const Params &P, int top)
+    {
+        oe_d2 = (uint32_t)min(P.o_del + P.e_del, top) * 0x10001u;
+        oe_i2 = (uint32_t)min(P.o_ins + P.e_ins, top) * 0x10001u;
+        ne_d2 = (uint32_t)(-P.e_del & 0xffff) * 0x10001u;
+        ne_i2 = (uint32_t)(-P.e_ins & 0xffff) * 0x10001u;
+        p0 = p1 = 0u;
     }
-    X.key = __viaddmax_u16x2(kb, X.j2, X.key);
-    X.j2 += (uint32_t)N * 0x10001u;
-    if (hh[N - 1] > 0xffffu) {
-        X.L = s + N;
-    } else {
-#pragma unroll
-        for (int k = 0; k < N - 1; ++k)
-            if (hh[k] > 0xffffu) X.L = s + k + 1;
+    __device__ __forceinline__ void rows(const Params &P, int t0, int t1)
+    {
+        const uint32_t mb = (uint32_t)(-P.b) & 0xffu, flip = ((uint32_t)P.a ^ mb) & 0xffu;
+        p0 = mb * 0x01010101u ^ (flip << (8 * t0));
+        p1 = mb * 0x01010101u ^ (flip << (8 * t1));
     }
-}
+};
 
+// 8-bit lanes (score bound at most 255).  Slot j: a selector in bits 0-15, E
+// in 16-23, H in 24-31.  The selector's nibbles are q_{j-1}, q_{j-1} | 8, 4 +
+// q_j, (4 + q_j) | 8 for a permute over both rows' scores, which it
+// sign-extends: row i+1's in the low half, row i's in the high one.  With N in
+// the queries (NM) the nibbles run over five codes, byte 4 being N's -1, so
+// each row's scores take a permute of their own and a third joins the halves
+// (1 M pairs of 250 bp reads with 0.1% N: 3.22 ms, 2.8 without N, 4.54 with
+// one row per pass).
 template <bool SYM, bool NM>
+struct RpLane8 {
+    static constexpr bool kN = NM;
+    static constexpr int kKey = 256;        // row key: H * kKey + column
+    RpK K;
+    uint32_t *S;
+    uint32_t k8, zm;
+
+    // The factors come from a run-time value so that the products stay
+    // multiplies (FMA pipe) instead of becoming shifts (integer pipe).
+    __device__ __forceinline__ RpLane8(const Params &P, uint32_t *slots) : K(P, 1023), S(slots), k8(P.k8), zm(P.k8 >> 1) {}
+
+    __device__ __forceinline__ uint16_t *eh(int j) const { return reinterpret_cast<uint16_t *>(S + j * 32) + 1; }
+    __device__ __forceinline__ void put(int j, int h, int e) const { *eh(j) = (uint16_t)(((uint32_t)h << 8) | (uint32_t)e); }
+    __device__ __forceinline__ void get(int j, int &h, int &e) const
+    {
+        const uint32_t w = S[j * 32];
+        h = (int)(w >> 24);
+        e = (int)((w >> 16) & 0xffu);
+    }
+    __device__ __forceinline__ bool nonzero(int j) const { return (S[j * 32] >> 16) != 0u; }
+    __device__ __forceinline__ int h_of(int j) const { return (int)(S[j * 32] >> 24); }
+
+    __device__ __forceinline__ uint32_t scores(uint32_t w) const
+    {
+        if (!NM) return prmt(K.p1, K.p0, w);
+        return prmt(prmt(K.p1, kNScore, w), prmt(K.p0, kNScore, w), 0x7610u);
+    }
+    __device__ __forceinline__ int score0(int j) const { return (int)scores(S[j * 32]) >> 16; }          // row i
+    __device__ __forceinline__ int score1(int j) const                                                    // row i + 1
+    {
+        return (int)(signed char)prmt(K.p1, kNScore, (S[j * 32] >> 8) & (NM ? 7u : 3u));
+    }
+
+    // Eq. 3, first row: H = h0 at column 0, max(0, h0 - o_ins - c*e_ins) after.
+    __device__ __forceinline__ void init(const Batch &B, const Params &P, const PairRec &R) const
+    {
+        const int n = R.n;
+        const uint8_t *qp = B.q + (R.q_off >> 2);
+        uint32_t cprev = 0;
+        for (int c = 0; c <= n; c += 4) {
+            const uint32_t byte = c < n ? __ldg(qp + (c >> 2)) : 0u;
+            const uint32_t nb = (NM && B.q_n && c < n) ? (uint32_t)__ldg(B.q_n + ((R.q_off + c) >> 3)) >> ((R.q_off + c) & 7) : 0u;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int j = c + k;
+                if (j <= n) {
+                    const uint32_t cj = j >= n ? 0u : NM && ((nb >> k) & 1u) ? 4u : (byte >> (2 * k)) & 3u;
+                    const int hv = j == 0 ? R.h0 : max(0, R.h0 - P.o_ins - j * P.e_ins);
+                    S[j * 32] = cj * 0x1100u + cprev * 0x11u + (NM ? 0x8080u : 0xc480u) + ((uint32_t)hv << 24);
+                    cprev = cj;
+                }
+            }
+        }
+    }
+    __device__ __forceinline__ void open(RpRow &X, int c0, int bnd1, int key_lo) const
+    {
+        X.hK = (uint32_t)bnd1 << 8;                                // low half used
+        X.key = (uint32_t)key_lo << 16;
+        X.j2 = ((uint32_t)(c0 + 1) << 16) | (uint32_t)c0;
+    }
+    __device__ __forceinline__ void close(const RpRow &X, int &key_lo, int &key_hi) const
+    {
+        key_lo = (int)(X.key >> 16);
+        key_hi = (int)(X.key & 0xffffu);
+    }
+
+    // N steps from step s: cells (i, s + k) and (i + 1, s + k - 1).  All N slots
+    // are read before the first is written back (step s + k writes slot s + k -
+    // 1, read before), so the loads' latency is paid once per block.  Within a
+    // block the keys hold the step's number; the block's first column is added
+    // once.  Blocks of 8: 4 or 16 steps run 4.5% slower and 0.6% faster on 250
+    // bp reads, 2% slower both on 151 bp reads.
+    template <int N>
+    __device__ __forceinline__ void steps(int s, RpRow &X) const
+    {
+        uint32_t *Sb = S + s * 32;
+        uint16_t *SEH = reinterpret_cast<uint16_t *>(Sb) + 1;      // E | H << 8 of slot s
+        uint32_t wv[N], hh[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) wv[k] = Sb[k * 32];
+        uint32_t kb = 0;
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const uint32_t Hd2 = prmt(X.hB, wv[k], 0x1712u);         // H(i, s-2) | H(i-1, s-1) << 16
+            const uint32_t Ed2 = prmt(X.EN, wv[k], 0x1612u);         // E(i+1, s-1) | E(i, s) << 16
+            // zero-diagonal rule: M = min(D + s, D * 128), D * 128 >= D + s for
+            // D >= 1 (match <= 127) and below 2^15 for D <= 255
+            const uint32_t M2 = __viaddmin_s16x2(Hd2, scores(wv[k]), Hd2 * zm);
+            const uint32_t h2 = __vimax3_s16x2(M2, Ed2, X.F);
+            const uint32_t Mi2 = sub_sat_h2(M2, K.oe_i2);
+            const uint32_t Md2 = SYM ? Mi2 : sub_sat_h2(M2, K.oe_d2);
+            const uint32_t EN2 = __viaddmax_s16x2(Ed2, K.ne_d2, Md2);
+            X.F = __viaddmax_s16x2(X.F, K.ne_i2, Mi2);
+            SEH[(k - 1) * 64] = (uint16_t)(X.hK + EN2);              // slot s-1 <- E(i+2, s-1), H(i+1, s-2)
+            X.hK = h2 * k8;
+            kb = k == 0 ? X.hK : __viaddmax_u16x2(X.hK, (uint32_t)k * 0x10001u, kb);
+            X.hB = X.hA;
+            X.hA = h2;
+            X.EN = EN2;
+            hh[k] = h2;
+        }
+        X.key = __viaddmax_u16x2(kb, X.j2, X.key);
+        X.j2 += (uint32_t)N * 0x10001u;
+        X.settle<N>(s, hh);
+    }
+};
+
+// 16-bit lanes up to a score bound of 2047 (kRp16Top), where sub_sat_h2 is
+// exact.  Slot j: E in the low half, H in the high one; the query's codes lie
+// beside the slots, a nibble each, eight to a word, so that one permute gives
+// a row's scores of four columns.  A block's keys are H * 8 + step in 16 bits
+// and join the row's 32-bit keys (H * 512 + column) once a block.
+constexpr int kRp16Top = 2047;
+__host__ __device__ constexpr int rp16_words(int nmax) { return nmax + 1 + nmax / 8 + 1; }
+
+template <bool SYM>
+struct RpLane16 {
+    static constexpr bool kN = false;
+    static constexpr int kKey = 512;
+    RpK K;
+    uint32_t *S, *Q;
+    uint32_t k3;                            // 2^3, a run-time value
+
+    __device__ __forceinline__ RpLane16(const Params &P, uint32_t *slots, int nmax)
+        : K(P, kRp16Top), S(slots), Q(slots + (nmax + 1) * 32), k3(P.k8 >> 5)
+    {
+    }
+
+    __device__ __forceinline__ void put(int j, int h, int e) const { S[j * 32] = ((uint32_t)h << 16) | (uint32_t)e; }
+    __device__ __forceinline__ void get(int j, int &h, int &e) const
+    {
+        const uint32_t w = S[j * 32];
+        h = (int)(w >> 16);
+        e = (int)(w & 0xffffu);
+    }
+    __device__ __forceinline__ bool nonzero(int j) const { return S[j * 32] != 0u; }
+    __device__ __forceinline__ int h_of(int j) const { return (int)(S[j * 32] >> 16); }
+    __device__ __forceinline__ int score(uint32_t p, int j) const
+    {
+        return (int)(signed char)prmt(p, 0u, (Q[(j >> 3) * 32] >> (4 * (j & 7))) & 3u);
+    }
+    __device__ __forceinline__ int score0(int j) const { return score(K.p0, j); }
+    __device__ __forceinline__ int score1(int j) const { return score(K.p1, j); }
+
+    __device__ __forceinline__ void init(const Batch &B, const Params &P, const PairRec &R) const
+    {
+        const int n = R.n;
+        const uint8_t *qp = B.q + (R.q_off >> 2);
+        for (int c = 0; c <= n; c += 8) {
+            uint32_t b = c < n ? __ldg(qp + (c >> 2)) : 0u;
+            if (c + 4 < n) b |= (uint32_t)__ldg(qp + (c >> 2) + 1) << 8;
+            uint32_t w = 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                w |= ((b >> (2 * k)) & 3u) << (4 * k);
+                const int j = c + k;
+                if (j <= n) put(j, j == 0 ? R.h0 : max(0, R.h0 - P.o_ins - j * P.e_ins), 0);
+            }
+            Q[(c >> 3) * 32] = w;
+        }
+    }
+    __device__ __forceinline__ void open(RpRow &X, int, int, int key_lo) const
+    {
+        X.k0 = key_lo;
+        X.k1 = 0;
+    }
+    __device__ __forceinline__ void close(const RpRow &X, int &key_lo, int &key_hi) const
+    {
+        key_lo = X.k0;
+        key_hi = X.k1;
+    }
+
+    template <int N>
+    __device__ __forceinline__ void steps(int s, RpRow &X) const
+    {
+        // codes of columns s-1 .. s+6 and s .. s+7, and their scores in rows i+1 and i
+        const uint32_t *q = Q + ((s - 1) >> 3) * 32;
+        const uint32_t q0 = q[0], q1 = q[32], sh = 4 * ((s - 1) & 7);
+        const uint32_t cl = __funnelshift_r(q0, q1, sh), ch = __funnelshift_r(cl, q1 >> sh, 4);
+        const uint32_t sl[2] = {prmt(K.p1, 0u, cl), N > 4 ? prmt(K.p1, 0u, cl >> 16) : 0u};
+        const uint32_t sg[2] = {prmt(K.p0, 0u, ch), N > 4 ? prmt(K.p0, 0u, ch >> 16) : 0u};
+        uint32_t *Sb = S + s * 32;
+        uint32_t wv[N], hh[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) wv[k] = Sb[k * 32];
+        uint32_t kb = 0;
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const uint32_t Hd2 = prmt(X.hB, wv[k], 0x7632u);         // H(i, s-2) | H(i-1, s-1) << 16
+            const uint32_t Ed2 = prmt(X.EN, wv[k], 0x5432u);         // E(i+1, s-1) | E(i, s) << 16
+            const uint32_t sc = prmt(sl[k >> 2], sg[k >> 2], 0xc480u + (uint32_t)(k & 3) * 0x1111u);
+            // zero-diagonal rule: M = min(D + s, z), z = 0 for D = 0 and above every score for D > 0
+            const uint32_t M2 = __viaddmin_s16x2(Hd2, sc, positive_h2(Hd2));
+            const uint32_t h2 = __vimax3_s16x2(M2, Ed2, X.F);
+            const uint32_t Mi2 = sub_sat_h2(M2, K.oe_i2);
+            const uint32_t Md2 = SYM ? Mi2 : sub_sat_h2(M2, K.oe_d2);
+            const uint32_t EN2 = __viaddmax_s16x2(Ed2, K.ne_d2, Md2);
+            X.F = __viaddmax_s16x2(X.F, K.ne_i2, Mi2);
+            Sb[(k - 1) * 32] = prmt(EN2, X.hA, 0x5410u);             // slot s-1 <- E(i+2, s-1), H(i+1, s-2)
+            const uint32_t h8 = h2 * k3;
+            kb = k == 0 ? h8 : __viaddmax_u16x2(h8, (uint32_t)k * 0x10001u, kb);
+            X.hB = X.hA;
+            X.hA = h2;
+            X.EN = EN2;
+            hh[k] = h2;
+        }
+        const int t0 = (int)(kb >> 16), t1 = (int)(kb & 0xffffu);
+        X.k0 = max(X.k0, t0 * 64 - (t0 & 7) * 63 + s);               // (t >> 3) * 512 + (t & 7) + s
+        X.k1 = max(X.k1, t1 * 64 - (t1 & 7) * 63 + s - 1);
+        X.settle<N>(s, hh);
+    }
+};
+
+// Extend one pair with two rows per pass on lane V.
+template <class Lane>
 __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, const Params &P, const PairRec &R,
-                                                            bsw_result_t *out, uint32_t *S)
+                                                            bsw_result_t *out, Lane &V)
 {
+    constexpr bool NM = Lane::kN;
+    constexpr int kKey = Lane::kKey;
     const int n = R.n, m = R.m, h0 = R.h0;
     const int wb = clip_band(P, n, R.w);
     const int e_del = P.e_del, e_ins = P.e_ins;
     const int oe_del = P.o_del + e_del, oe_ins = P.o_ins + e_ins;
-    // Zero-diagonal rule: M = min(D + s, D * 128), D * 128 >= D + s for D >= 1
-    // (match <= 127) and below 2^15 for D <= 255.  The factors come from a
-    // run-time value so that the products stay multiplies (FMA pipe) instead of
-    // becoming shifts (integer pipe).
-    RpK K;
-    K.k8 = P.k8;
-    K.zm = P.k8 >> 1;
-    // opening costs above every M (at most 255) act alike
-    K.oe_d2 = (uint32_t)min(oe_del, 1023) * 0x10001u;
-    K.oe_i2 = (uint32_t)min(oe_ins, 1023) * 0x10001u;
-    K.ne_d2 = (uint32_t)(-e_del & 0xffff) * 0x10001u;
-    K.ne_i2 = (uint32_t)(-e_ins & 0xffff) * 0x10001u;
-
-    // Eq. 3, first row, and the selectors: slot j = q_j * 0x1100 + q_{j-1} * 0x11
-    // + 0x8480 (nibbles q_{j-1}, q_{j-1} | 8, 4 + q_j, (4 + q_j) | 8), or without
-    // the 4's with N codes.
-    constexpr uint32_t kSel = NM ? 0x8080u : 0xc480u;
-    const int64_t q_off = R.q_off;
-    const uint8_t *qp = B.q + (q_off >> 2);
-    uint32_t cprev = 0;
-    for (int c = 0; c <= n; c += 4) {
-        const uint32_t byte = c < n ? __ldg(qp + (c >> 2)) : 0u;
-        const uint32_t nb = (NM && B.q_n && c < n) ? (uint32_t)__ldg(B.q_n + ((q_off + c) >> 3)) >> ((q_off + c) & 7) : 0u;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int j = c + k;
-            if (j <= n) {
-                const uint32_t cj = j >= n ? 0u : NM && ((nb >> k) & 1u) ? 4u : (byte >> (2 * k)) & 3u;
-                const int hv = j == 0 ? h0 : max(0, h0 - P.o_ins - j * e_ins);
-                S[j * 32] = cj * 0x1100u + cprev * 0x11u + kSel + ((uint32_t)hv << 24);
-                cprev = cj;
-            }
-        }
-    }
+    V.init(B, P, R);
     const uint8_t *tn = NM ? B.t_n : nullptr;
     const int64_t t_off = R.t_off;
     const uint8_t *tp = B.t + (t_off >> 2);
@@ -613,10 +790,6 @@ __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, cons
         if (NM && tn) v |= (((uint32_t)__ldg(tn + ((t_off + i) >> 3)) >> ((t_off + i) & 7)) & 15u) << 8;
         return v;
     };
-    const uint32_t mb8 = (uint32_t)(-P.b) & 0xffu;
-    const uint32_t mis4 = mb8 * 0x01010101u;
-    const uint32_t flip = ((uint32_t)P.a ^ mb8) & 0xffu;
-    uint16_t *SEH = reinterpret_cast<uint16_t *>(reinterpret_cast<uint8_t *>(S) + 2);     // E | H << 8 of slot 0
 
     int lo = 0, hi = n;
     int best = h0, bi = -1, bj = -1, gbest = -1, gi = -1, moff = 0;
@@ -628,10 +801,9 @@ __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, cons
             tnext = i + 4 < m ? t_rows(i + 4) : 0u;
         }
         const int tb0 = (tbyte >> (2 * (i & 3))) & 3, tb1 = (tbyte >> (2 * (i & 3) + 2)) & 3;
-        K.p0 = mis4 ^ (flip << (8 * tb0));       // row i: byte c = s(t_i, c)
-        K.p1 = mis4 ^ (flip << (8 * tb1));       // row i+1
-        if (NM && ((tbyte >> (8 + (i & 3))) & 1u)) K.p0 = kNScore;
-        if (NM && ((tbyte >> (9 + (i & 3))) & 1u)) K.p1 = kNScore;
+        V.K.rows(P, tb0, tb1);
+        if (NM && ((tbyte >> (8 + (i & 3))) & 1u)) V.K.p0 = kNScore;
+        if (NM && ((tbyte >> (9 + (i & 3))) & 1u)) V.K.p1 = kNScore;
         const bool single = i + 1 == m;
         lo = max(lo, i - wb);
         hi = min(min(hi, i + wb + 1), n);
@@ -643,20 +815,20 @@ __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, cons
         int lo1 = hi, c0 = -1;
         bool found = false;
         for (int s = lo; s < hi; ++s) {
-            const uint32_t wv = S[s * 32];
-            const int d = (int)(wv >> 24), e = (int)((wv >> 16) & 0xffu);
-            const int M = d > 0 ? d + ((int)rp_scores<NM>(K, wv) >> 16) : 0;
+            int d, e;
+            V.get(s, d, e);
+            const int M = d > 0 ? d + V.score0(s) : 0;
             const int h = __vimax3_s32(M, e, f);
             const int en = __viaddmax_s32_relu(e, -e_del, M - oe_del);
             f = __viaddmax_s32_relu(f, -e_ins, M - oe_ins);
-            key_lo = max(key_lo, h * 256 + s);
+            key_lo = max(key_lo, h * kKey + s);
             if (h > 0) Lp = s + 1;
             if (!found && (hprev | en)) { found = true; lo1 = s; }
             hprev2 = hprev; hprev = h; en_last = en;
             if (!single && found && s >= max(lo1, i + 1 - wb)) { c0 = s; break; }
         }
         if (single) {                                        // the last row of an odd count
-            const int rm = key_lo >> 8, rj = key_lo & 255;
+            const int rm = key_lo / kKey, rj = key_lo % kKey;
             if (hi > lo) ncell += (unsigned)(hi - lo);
             if (max(lo, hi) == n) {
                 const int hl = hi > lo ? hprev : hl0;
@@ -678,19 +850,17 @@ __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, cons
         RpRow X;
         X.hA = (uint32_t)bnd1 | ((uint32_t)hprev << 16);
         X.hB = (uint32_t)hprev2 << 16;                             // high half used
-        X.hK = (uint32_t)bnd1 << 8;                                // low half used
         X.EN = (uint32_t)en_last << 16;                            // high half used
         X.F = (uint32_t)f << 16;
-        X.key = (uint32_t)key_lo << 16;
         X.L = Lp;
-        X.j2 = ((uint32_t)(c0 + 1) << 16) | (uint32_t)c0;
+        V.open(X, c0, bnd1, key_lo);
         {
             int s = c0 + 1;
-            for (; s + 8 <= hi; s += 8) rp_steps<8, SYM, NM>(S, s, K, X);
+            for (; s + 8 <= hi; s += 8) V.template steps<8>(s, X);
             const int rest = max(hi - s, 0);                        // c0 can lie past hi: no steps
-            if (rest & 4) { rp_steps<4, SYM, NM>(S, s, K, X); s += 4; }
-            if (rest & 2) { rp_steps<2, SYM, NM>(S, s, K, X); s += 2; }
-            if (rest & 1) rp_steps<1, SYM, NM>(S, s, K, X);
+            if (rest & 4) { V.template steps<4>(s, X); s += 4; }
+            if (rest & 2) { V.template steps<2>(s, X); s += 2; }
+            if (rest & 1) V.template steps<1>(s, X);
         }
         int Hi1, Hi2, Ei1, ce, fh, hlh;                            // row i's last values; row i+1's state
         if (hi > c0 + 1) {
@@ -701,12 +871,12 @@ __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, cons
             Hi1 = hprev; Hi2 = hprev2; Ei1 = en_last;
             ce = c0; fh = 0; hlh = bnd1;
         }
-        key_lo = (int)(X.key >> 16);
-        int key_hi = (int)(X.key & 0xffffu);
+        int key_hi;
+        V.close(X, key_lo, key_hi);
 
         // Row i: Section V-D's decisions.
         {
-            const int rm = key_lo >> 8, rj = key_lo & 255;
+            const int rm = key_lo / kKey, rj = key_lo % kKey;
             if (hi > lo) ncell += (unsigned)(hi - lo);
             if (max(lo, hi) == n) {
                 const int hl = hi > lo ? Hi1 : hl0;
@@ -727,25 +897,24 @@ __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, cons
         const int i1 = i + 1;
         const int hi1 = min(min(Lp + 2, n), i1 + wb + 1);
         for (int c = ce; c < hi1; ++c) {
-            const uint32_t wc = S[c * 32];
             int d, e;
             if (c == hi - 1) { d = Hi2; e = Ei1; }
             else if (c == hi) { d = Hi1; e = 0; }
-            else { d = (int)(wc >> 24); e = (int)((wc >> 16) & 0xffu); }   // past row i: the slot as it stands
-            const int M = d > 0 ? d + (int)(signed char)prmt(K.p1, kNScore, (wc >> 8) & (NM ? 7u : 3u)) : 0;
+            else V.get(c, d, e);                                       // past row i: the slot as it stands
+            const int M = d > 0 ? d + V.score1(c) : 0;
             const int h = __vimax3_s32(M, e, fh);
             const int en = __viaddmax_s32_relu(e, -e_del, M - oe_del);
             fh = __viaddmax_s32_relu(fh, -e_ins, M - oe_ins);
-            SEH[c * 64] = (uint16_t)(((uint32_t)hlh << 8) | (uint32_t)en);
-            key_hi = max(key_hi, h * 256 + c);
+            V.put(c, hlh, en);
+            key_hi = max(key_hi, h * kKey + c);
             hlh = h;
         }
-        if (hi1 >= ce && hi1 > c0) SEH[hi1 * 64] = (uint16_t)((uint32_t)hlh << 8);   // row end, E = 0
+        if (hi1 >= ce && hi1 > c0) V.put(hi1, hlh, 0);               // row end, E = 0
         {
-            const int rm = key_hi >> 8, rj = key_hi & 255;
+            const int rm = key_hi / kKey, rj = key_hi % kKey;
             if (hi1 > c0) ncell += (unsigned)(hi1 - c0);
             if (max(c0, hi1) == n) {
-                const int hl = hi1 > c0 ? (int)(S[hi1 * 32] >> 24) : bnd1;
+                const int hl = hi1 > c0 ? V.h_of(hi1) : bnd1;
                 if (hl >= gbest) gi = i1;
                 gbest = max(gbest, hl);
             }
@@ -759,12 +928,12 @@ __device__ __forceinline__ unsigned long long inter_pair_rp(const Batch &B, cons
                 if (drop > P.zdrop) break;
             }
         }
-        for (int k = hi1 + 1; k <= hi; ++k) SEH[k * 64] = 0;       // row i's zeros past row i+1's end
+        for (int k = hi1 + 1; k <= hi; ++k) V.put(k, 0, 0);        // row i's zeros past row i+1's end
         int k = c0;                                                // rule c on row i+1
-        while (k < hi1 && !slot_nonzero<true>(S[k * 32])) ++k;
+        while (k < hi1 && !V.nonzero(k)) ++k;
         lo = k;
         k = hi1;
-        while (k >= lo && !slot_nonzero<true>(S[k * 32])) --k;
+        while (k >= lo && !V.nonzero(k)) --k;
         hi = min(k + 2, n);
     }
     store_result(out, best, bj + 1, bi + 1, gi + 1, gbest, moff);
@@ -797,11 +966,12 @@ __device__ __forceinline__ PairRec pair_rec(const Batch &B, const Params &P, con
 // bitmaps.
 // Launch bounds: blocks have at most 4 warps, and 6 of them at most share an
 // SM's registers: up to 85 a thread, which the steps' loads in flight use (4 M
-// pairs of 250 bp reads: 10.85 ms; 5 blocks 11.04, 4 blocks 11.19, 64 registers
-// 11.18; shared memory holds 12 warps of the 128-base class).  With N bases the
-// two more permutes a step want 5 (1 M pairs: 3.15 ms against 3.25).
+// pairs of 250 bp reads: 10.74 ms; before the lanes had a class of their own 6,
+// 5 and 4 blocks took 10.85, 11.04 and 11.19, 64 registers 11.18; with N, 1 M
+// pairs: 3.22, 3.25 and 3.24).  Shared memory holds 12 warps of the 128-base
+// class.
 template <bool SYM, bool NM>
-__global__ void __launch_bounds__(128, NM ? 5 : 6) k_rows2(Batch B, Params P, Work W, int cls, int nmax)
+__global__ void __launch_bounds__(128, 6) k_rows2(Batch B, Params P, Work W, int cls, int nmax)
 {
     extern __shared__ uint32_t smem[];
     const int lane = threadIdx.x & 31;
@@ -813,7 +983,8 @@ __global__ void __launch_bounds__(128, NM ? 5 : 6) k_rows2(Batch B, Params P, Wo
         const int idx = (g << 5) + lane;
         if (idx < count) {
             const int p = W.order[start + idx];
-            cells += inter_pair_rp<SYM, NM>(B, P, pair_rec(B, P, W, start + idx, p), &B.out[p], S);
+            RpLane8<SYM, NM> V(P, S);
+            cells += inter_pair_rp(B, P, pair_rec(B, P, W, start + idx, p), &B.out[p], V);
         }
         __syncwarp();
     }
@@ -821,14 +992,47 @@ __global__ void __launch_bounds__(128, NM ? 5 : 6) k_rows2(Batch B, Params P, Wo
     if (lane == 0 && cells) atomicAdd(W.cells, cells);
 }
 
-// Persistent kernel with one row at a time: the 16-bit classes, and the 8-bit
-// ones where k_rows2 does not apply (rows2_ok), which take batches with N too.
-template <int NMAX, bool U8>
-__global__ void __launch_bounds__(128, 5) k_inter(Batch B, Params P, Work W, int cls)
+// Persistent kernel of a 16-bit class: two rows per instruction up to a score
+// bound of kRp16Top, one row at a time above (and for gap costs that do not
+// fit the halves), where scores up to 32767 stay in the lane.  1 M pairs of 250
+// bp reads with match 2: 7.32 ms with one row at a time (ALU pipe 65% busy, 8
+// warps per SM), 4.03 ms so; at 4, 5 and 6 blocks of launch bounds 4.04, 4.03
+// and 4.08.
+template <bool SYM>
+__global__ void __launch_bounds__(128, 5) k_rows2_16(Batch B, Params P, Work W, int cls, int nmax)
 {
     extern __shared__ uint32_t smem[];
     const int lane = threadIdx.x & 31;
-    uint32_t *S = smem + (threadIdx.x >> 5) * ((NMAX + 1) * 32) + lane;
+    uint32_t *S = smem + (threadIdx.x >> 5) * (rp16_words(nmax) * 32) + lane;
+    const int start = W.cls_start[cls], count = W.cls_count[cls];
+    const int ngroups = (count + 31) >> 5;
+    const bool fits = P.o_del + P.e_del <= 30000 && P.o_ins + P.e_ins <= 30000;
+    unsigned long long cells = 0;
+    for (int g; (g = next_group(W, cls, lane, ngroups)) >= 0;) {
+        const int idx = (g << 5) + lane;
+        if (idx < count) {
+            const int p = W.order[start + idx];
+            const PairRec R = pair_rec(B, P, W, start + idx, p);
+            if (fits && (long long)R.h0 + (long long)P.a * min(R.n, R.m) <= kRp16Top) {
+                RpLane16<SYM> V(P, S, nmax);
+                cells += inter_pair_rp(B, P, R, &B.out[p], V);
+            } else {
+                cells += inter_pair<false, false>(B, P, W, p, R, S, nmax);
+            }
+        }
+        __syncwarp();
+    }
+    for (int d = 16; d > 0; d >>= 1) cells += __shfl_xor_sync(kFull, cells, d);
+    if (lane == 0 && cells) atomicAdd(W.cells, cells);
+}
+
+// Persistent kernel of an 8-bit class with one row at a time, where k_rows2
+// does not apply (rows2_ok); it takes batches with N too.
+__global__ void __launch_bounds__(128, 5) k_rows1(Batch B, Params P, Work W, int cls, int nmax)
+{
+    extern __shared__ uint32_t smem[];
+    const int lane = threadIdx.x & 31;
+    uint32_t *S = smem + (threadIdx.x >> 5) * ((nmax + 1) * 32) + lane;
     const int start = W.cls_start[cls], count = W.cls_count[cls];
     const int ngroups = (count + 31) >> 5;
     unsigned long long cells = 0;
@@ -836,7 +1040,7 @@ __global__ void __launch_bounds__(128, 5) k_inter(Batch B, Params P, Work W, int
         const int idx = (g << 5) + lane;
         if (idx < count) {
             const int p = W.order[start + idx];
-            cells += inter_pair<NMAX, U8, U8>(B, P, W, p, pair_rec(B, P, W, start + idx, p), S);
+            cells += inter_pair<true, true>(B, P, W, p, pair_rec(B, P, W, start + idx, p), S, nmax);
         }
         __syncwarp();
     }
@@ -2074,49 +2278,50 @@ Plan default_plan()
 
 namespace {
 
-// Resident blocks per SM of each per-thread class's kernels with 1, 2 and 4
-// warps per block, set by prepare_kernels.
-int g_inter_blocks[12][3];      // k_inter
+// Resident blocks per SM of the per-thread kernels with 1, 2 and 4 warps per
+// block, by class bound, set by prepare_kernels.
+int g_rows1_blocks[8][3];       // k_rows1
 int g_rows2_blocks[2][8][3];    // k_rows2, without and with N
+int g_rows16_blocks[4][3];      // k_rows2_16
 
 int warps_index(int warps) { return warps <= 1 ? 0 : warps == 2 ? 1 : 2; }
 
-// A slot column of 32-bit words per lane, for either per-thread kernel.
-size_t inter_smem(int nmax, int warps) { return (size_t)warps * (nmax + 1) * 32 * 4; }
-template <int NMAX, bool U8> constexpr int inter_index()
-{
-    return U8 ? (NMAX >= 256 ? 0 : NMAX >= 224 ? 1 : NMAX >= 192 ? 2 : NMAX >= 160 ? 3 : NMAX >= 128 ? 4 : NMAX >= 96 ? 5
-                 : NMAX >= 64 ? 6 : 7)
-              : 8 + (NMAX >= 256 ? 0 : NMAX >= 128 ? 1 : NMAX >= 64 ? 2 : 3);
-}
+// Shared memory of a block: a column of 32-bit words per lane.
+size_t rows_smem(int words, int warps) { return (size_t)warps * words * 32 * 4; }
 
-// The kernel's shared-memory limit, and its resident blocks with queries up
-// to nmax bases.
+// A per-thread kernel's shared-memory limit (words_max per lane), and its
+// resident blocks at `words` per lane.
 template <class K>
-cudaError_t prepare_slots(K *kernel, int nmax, int *blocks)
+cudaError_t prepare_rows(K *kernel, int words_max, int words, int *blocks)
 {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)inter_smem(kShortMax, 4));
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows_smem(words_max, 4));
     for (int wi = 0; wi < 3 && e == cudaSuccess; ++wi) {
         int nb = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, 32 << wi, inter_smem(nmax, 1 << wi));
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, 32 << wi, rows_smem(words, 1 << wi));
         blocks[wi] = nb > 0 ? nb : 1;
     }
     return e;
 }
 
-// The 8-bit instantiations of k_inter are the N-aware ones (they take batches
-// without N too); split gap costs need no more of an SM than equal ones.
-template <int NMAX, bool U8>
-cudaError_t prepare_inter()
+// Split gap costs need no more of an SM than equal ones, so the equal ones'
+// block counts serve both.
+cudaError_t prepare_per_thread()
 {
-    constexpr int c = inter_index<NMAX, U8>();
-    cudaError_t e = prepare_slots(k_inter<NMAX, U8>, NMAX, g_inter_blocks[c]);
-    if (e != cudaSuccess || !U8) return e;
+    cudaError_t e = cudaSuccess;
+    const int top = kShortMax + 1, top16 = rp16_words(kShortMax);
     int unused[3];
-    if ((e = prepare_slots(k_rows2<false, false>, NMAX, unused)) != cudaSuccess) return e;
-    if ((e = prepare_slots(k_rows2<false, true>, NMAX, unused)) != cudaSuccess) return e;
-    if ((e = prepare_slots(k_rows2<true, false>, NMAX, g_rows2_blocks[0][c & 7])) != cudaSuccess) return e;
-    return prepare_slots(k_rows2<true, true>, NMAX, g_rows2_blocks[1][c & 7]);
+    for (int c = 0; c < 8 && e == cudaSuccess; ++c) {
+        const int words = kU8Nmax[c] + 1;
+        if ((e = prepare_rows(k_rows1, top, words, g_rows1_blocks[c])) != cudaSuccess) return e;
+        if ((e = prepare_rows(k_rows2<true, false>, top, words, g_rows2_blocks[0][c])) != cudaSuccess) return e;
+        e = prepare_rows(k_rows2<true, true>, top, words, g_rows2_blocks[1][c]);
+    }
+    for (int c = 0; c < 4 && e == cudaSuccess; ++c)
+        e = prepare_rows(k_rows2_16<true>, top16, rp16_words(kI16Nmax[c]), g_rows16_blocks[c]);
+    if (e == cudaSuccess) e = prepare_rows(k_rows2<false, false>, top, top, unused);
+    if (e == cudaSuccess) e = prepare_rows(k_rows2<false, true>, top, top, unused);
+    if (e == cudaSuccess) e = prepare_rows(k_rows2_16<false>, top16, top16, unused);
+    return e;
 }
 
 // Whether the 8-bit classes run two rows per instruction: the gap costs fit
@@ -2126,18 +2331,19 @@ bool rows2_ok(const Params &P)
     return !(P.flags & BSW_FORCE_I8) && P.o_del + P.e_del <= 30000 && P.o_ins + P.e_ins <= 30000;
 }
 
-template <int NMAX, bool U8>
-cudaError_t launch_inter(const Batch &B, const Params &P, const Work &W, int cls, cudaStream_t st, int sms, int warps)
+bool symmetric(const Params &P) { return P.o_del == P.o_ins && P.e_del == P.e_ins; }
+
+// 8-bit class cls (0-7), one pair per thread.
+cudaError_t launch_rows8(const Batch &B, const Params &P, const Work &W, int cls, cudaStream_t st, int sms, int warps)
 {
-    constexpr int c = inter_index<NMAX, U8>();
-    const size_t smem = inter_smem(NMAX, warps);
-    if (U8 && rows2_ok(P)) {
-        const bool nm = B.q_n || B.t_n, sym = P.o_del == P.o_ins && P.e_del == P.e_ins;
-        const int blocks = sms * g_rows2_blocks[nm][c & 7][warps_index(warps)];
+    const int nmax = kU8Nmax[cls], wi = warps_index(warps);
+    const size_t smem = rows_smem(nmax + 1, warps);
+    if (rows2_ok(P)) {
+        const bool nm = B.q_n || B.t_n, sym = symmetric(P);
         auto *k = nm ? (sym ? k_rows2<true, true> : k_rows2<false, true>) : (sym ? k_rows2<true, false> : k_rows2<false, false>);
-        k<<<blocks, warps * 32, smem, st>>>(B, P, W, cls, NMAX);
+        k<<<sms * g_rows2_blocks[nm][cls][wi], warps * 32, smem, st>>>(B, P, W, cls, nmax);
     } else {
-        k_inter<NMAX, U8><<<sms * g_inter_blocks[c][warps_index(warps)], warps * 32, smem, st>>>(B, P, W, cls);
+        k_rows1<<<sms * g_rows1_blocks[cls][wi], warps * 32, smem, st>>>(B, P, W, cls, nmax);
     }
     return cudaGetLastError();
 }
@@ -2184,7 +2390,7 @@ cudaError_t launch_u8(const Batch &B, const Params &P, const Work &W, int cls, c
         k_inter2<N2><<<blocks, inter2_warps<N2>() * 32, inter2_smem<N2>(), st>>>(B, P, W, cls);
         return cudaGetLastError();
     }
-    return launch_inter<NMAX, true>(B, P, W, cls, st, sms, L.inter_warps);
+    return launch_rows8(B, P, W, cls, st, sms, L.inter_warps);
 }
 
 // Ring size for the context's band: the smallest power of two >= 2*w + 3,
@@ -2242,10 +2448,12 @@ cudaError_t cls_u8(const Batch &B, const Params &P, const Work &W, int c, cudaSt
     return launch_u8<NMAX>(B, P, W, c, st, sms, L);
 }
 
-template <int NMAX>
 cudaError_t cls_i16(const Batch &B, const Params &P, const Work &W, int c, cudaStream_t st, int sms, int, const Plan &L)
 {
-    return launch_inter<NMAX, false>(B, P, W, c, st, sms, L.inter_warps);
+    const int nmax = kI16Nmax[c - 8], warps = L.inter_warps;
+    auto *k = symmetric(P) ? k_rows2_16<true> : k_rows2_16<false>;
+    k<<<sms * g_rows16_blocks[c - 8][warps_index(warps)], warps * 32, rows_smem(rp16_words(nmax), warps), st>>>(B, P, W, c, nmax);
+    return cudaGetLastError();
 }
 
 cudaError_t cls_w16(const Batch &B, const Params &P, const Work &W, int c, cudaStream_t st, int sms, int wblocks,
@@ -2271,7 +2479,7 @@ cudaError_t cls_cta(const Batch &B, const Params &P, const Work &W, int c, cudaS
 
 constexpr ClassLaunch kClassLaunch[kNumClass + 1] = {
     cls_u8<256>, cls_u8<224>, cls_u8<192>, cls_u8<160>, cls_u8<128>, cls_u8<96>, cls_u8<64>, cls_u8<32>,
-    cls_i16<256>, cls_i16<128>, cls_i16<64>, cls_i16<32>, cls_cta, cls_w16, cls_w32, cls_w32};
+    cls_i16, cls_i16, cls_i16, cls_i16, cls_cta, cls_w16, cls_w32, cls_w32};
 
 // Launch order of the classes in the forked path and the side stream of each:
 // the longest work first (block-per-pair pairs, then the long 8-bit classes).
@@ -2380,18 +2588,7 @@ cudaError_t prepare_kernels(int sms)
     if ((e = cudaFuncSetAttribute(k_plain<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingSmemMax)) != cudaSuccess)
         return e;
     if ((e = prepare_x2(sms)) != cudaSuccess) return e;
-    if ((e = prepare_inter<256, true>()) != cudaSuccess) return e;
-    if ((e = prepare_inter<192, true>()) != cudaSuccess) return e;
-    if ((e = prepare_inter<128, true>()) != cudaSuccess) return e;
-    if ((e = prepare_inter<96, true>()) != cudaSuccess) return e;
-    if ((e = prepare_inter<64, true>()) != cudaSuccess) return e;
-    if ((e = prepare_inter<224, true>()) != cudaSuccess) return e;
-    if ((e = prepare_inter<32, true>()) != cudaSuccess) return e;
-    if ((e = prepare_inter<160, true>()) != cudaSuccess) return e;
-    if ((e = prepare_inter<256, false>()) != cudaSuccess) return e;
-    if ((e = prepare_inter<128, false>()) != cudaSuccess) return e;
-    if ((e = prepare_inter<64, false>()) != cudaSuccess) return e;
-    if ((e = prepare_inter<32, false>()) != cudaSuccess) return e;
+    if ((e = prepare_per_thread()) != cudaSuccess) return e;
     if ((e = prepare_inter2<128>()) != cudaSuccess) return e;
     if ((e = prepare_inter2<64>()) != cudaSuccess) return e;
     return prepare_inter2<32>();
