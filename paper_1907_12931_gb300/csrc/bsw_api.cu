@@ -1790,7 +1790,8 @@ int bsw_fm_build(bsw_ctx_t *ctx, const uint8_t *ref, int64_t n)
     if (rc != BSW_OK) return rc;
     cudaError_t e;
     if ((e = cudaMemcpy(ctx->fmbuf.p, ft.occ.data(), bt, cudaMemcpyHostToDevice)) != cudaSuccess) return cuda_rc(e);
-    ctx->fm_t = FmDev{(const FmEntry *)ctx->fmbuf.p, ft.n, ft.primary, {ft.C[0], ft.C[1], ft.C[2], ft.C[3], ft.C[4]}};
+    ctx->fm_t = FmDev{(const FmEntry *)ctx->fmbuf.p, (uint32_t)ft.primary,
+                      {(uint32_t)ft.C[0], (uint32_t)ft.C[1], (uint32_t)ft.C[2], (uint32_t)ft.C[3], (uint32_t)ft.C[4]}};
     ctx->fm_ready = true;
     return BSW_OK;
 }
@@ -1823,13 +1824,23 @@ int bsw_smem_n(bsw_ctx_t *ctx, int64_t n_reads, const uint8_t *reads, const uint
         }
         size_t o = 0;
         auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes, 256); return r; };
+        const int64_t groups = (n_reads + 31) / 32;
+        const int starts_cap = smem_starts_cap(lmax);
         const size_t o_reads = take((size_t)read_bytes), o_roff = take(8 * (size_t)n_reads),
                      o_rlen = take(4 * (size_t)n_reads), o_cnt = take(8 * (size_t)n_reads),
                      o_first = take(8 * (size_t)n_reads), o_ids = take(4 * (size_t)n_reads), o_nids = take(4),
-                     o_next = take(4), o_keep = take(sizeof(bsw_smem_t) * kSmemKeep * (size_t)n_reads),
+                     o_next = take(4), o_keep = take(sizeof(uint4) * kSmemKeep * (size_t)n_reads),
                      o_rn = take(reads_n ? (size_t)((read_bytes + 1) / 2) : 0),
                      o_out = take(sizeof(bsw_smem_t) * (size_t)std::max<int64_t>(out_cap, 1));
-        int rc = ctx->smemio.reserve(o, ctx->budget);
+        // the search starts of as many groups at a time as the budget holds
+        int64_t chunk = groups;
+        size_t o_starts = o, o_nst = 0;
+        int rc;
+        for (;; chunk = (chunk + 1) / 2) {
+            o_nst = align_up(o_starts + 4 * (size_t)chunk * (size_t)starts_cap, 256);
+            rc = ctx->smemio.reserve(o_nst + 4 * (size_t)chunk, ctx->budget);
+            if (rc != BSW_EBUDGET || chunk == 1) break;
+        }
         if (rc != BSW_OK) return rc;
         uint8_t *d = ctx->smemio.p;
         cudaStream_t st = ctx->sync.S.main;
@@ -1847,8 +1858,9 @@ int bsw_smem_n(bsw_ctx_t *ctx, int64_t n_reads, const uint8_t *reads, const uint
         int32_t *ids = (int32_t *)(d + o_ids);
         uint32_t *nids = (uint32_t *)(d + o_nids);
         int64_t *dfirst = (int64_t *)(d + o_first);
-        const SmemWork W{(int64_t *)(d + o_cnt), (bsw_smem_t *)(d + o_keep), dfirst, (bsw_smem_t *)(d + o_out),
-                         (uint32_t *)(d + o_next), nids, ids};
+        const SmemWork W{(int64_t *)(d + o_cnt), (uint4 *)(d + o_keep), dfirst, (bsw_smem_t *)(d + o_out),
+                         (uint32_t *)(d + o_next), nids, ids, (uint32_t *)(d + o_starts),
+                         (uint32_t *)(d + o_nst), starts_cap};
         auto global_lists = [&](int64_t n_ids, BiIv **lists) -> int {      // lmax + 1 entries hold any list
             const int r2 = ctx->smemscratch.reserve(sizeof(BiIv) * (size_t)n_ids * (size_t)(lmax + 1), ctx->budget);
             *lists = (BiIv *)ctx->smemscratch.p;
@@ -1857,7 +1869,7 @@ int bsw_smem_n(bsw_ctx_t *ctx, int64_t n_reads, const uint8_t *reads, const uint
 
         // One search pass: counts, and the records of reads with few; reads whose
         // lists overflow shared memory are searched with lists in global memory.
-        if ((e = launch_smem_store(R, ctx->fm_t, min_len, W, st, ctx->sms)) != cudaSuccess ||
+        if ((e = launch_smem_store(R, ctx->fm_t, min_len, W, chunk, st, ctx->sms)) != cudaSuccess ||
             (e = cudaMemcpyAsync(ctx->h_status, nids, 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
             (e = cudaStreamSynchronize(st)) != cudaSuccess)
             return cuda_rc(e);

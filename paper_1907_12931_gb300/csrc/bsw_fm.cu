@@ -16,17 +16,22 @@
 // subtracted.
 //
 // SMEMs of a read X (Li 2012; Algorithm 4): from a position x, extend X[x]
-// forward base by base, keeping the bi-interval each time its size is about to
-// shrink (one per distinct occurrence count, longest match last); then extend
+// forward base by base, keeping the match each time its number of occurrences
+// is about to shrink (one per distinct count, longest match last); then extend
 // those matches backward one base at a time, longest first.  A match that can
 // no longer be extended while no longer one survives at that base is an SMEM.
 // The next x is the end of the longest match from x; every SMEM holds exactly
-// one of the visited x.  One thread takes one read at a time; its list of
-// bi-intervals lives in shared memory (kListCap entries), and a read whose
-// list would grow beyond that is finished by a launch with lists in global
-// memory.  One pass keeps up to kSmemKeep records per read in a scratch
-// buffer; after the host's prefix sum a gather puts them in place, and the
-// rare reads with more are searched again, writing in place.
+// one of the visited x.
+//
+// The starts x depend on the forward searches alone, so the search is cut in
+// two kernels whose lanes do the same work at the same time: k_smem_scan takes
+// a read per lane, one base per step, and notes the starts; k_smem_store takes a
+// start per lane and does its forward and backward pass.  A read with more than
+// kListCap matches in one list is finished by a launch with lists in global
+// memory (k_smem_global), where a lane does a whole read.  One pass keeps up to
+// kSmemKeep records per read in a scratch buffer; after the host's prefix sum a
+// gather sorts them into place, and the rare reads with more are searched
+// again, writing in place.
 #include <cuda_runtime.h>
 #include <climits>
 #include <cstdint>
@@ -44,7 +49,7 @@ void fm_from_sa(const uint8_t *text, int64_t n, const int32_t *sa, FmHost &out)
 {
     const int64_t N = n + 1;
     out.n = N;
-    out.occ.assign((size_t)(N / 32 + 1), FmEntry{{0, 0, 0, 0}, 0, 0});
+    out.occ.assign((size_t)(N / 32 + 1), FmEntry{{0, 0, 0, 0}, 0, 0, {0, 0}});
     uint32_t cnt[4] = {0, 0, 0, 0};
     out.primary = -1;
     for (int64_t i = 0; i < N; ++i) {
@@ -60,7 +65,9 @@ void fm_from_sa(const uint8_t *text, int64_t n, const int32_t *sa, FmHost &out)
             b = text[sa[i] - 1];
             ++cnt[b];
         }
-        out.occ[(size_t)(i >> 5)].bwt |= (uint64_t)b << (2 * (i & 31));
+        FmEntry &e = out.occ[(size_t)(i >> 5)];
+        e.lo |= (uint32_t)(b & 1) << (i & 31);
+        e.hi |= (uint32_t)(b >> 1) << (i & 31);
     }
     if ((N & 31) == 0) {
         FmEntry &e = out.occ[(size_t)(N >> 5)];
@@ -68,98 +75,127 @@ void fm_from_sa(const uint8_t *text, int64_t n, const int32_t *sa, FmHost &out)
     }
     out.C[0] = 1;                                         // the terminator sorts first
     for (int c = 0; c < 4; ++c) out.C[c + 1] = out.C[c] + cnt[c];
+    for (FmEntry &e : out.occ)                            // the first row of each base, so that a lookup gives rows
+        for (int c = 0; c < 4; ++c) e.cnt[c] += (uint32_t)out.C[c];
 }
 
 // --------------------------------------------------------------------- device
 
 namespace {
 
-// Occurrences of each base in BWT[0, i) (Algorithm 1, all four from one bucket).
-__device__ __forceinline__ void occ4(const FmDev &F, uint32_t i, uint32_t o[4])
+// A bucket of O in registers, by one 256-bit load: the lanes of a warp look up
+// rows all over the table, so a load costs a pass of the L1 per lane, and a
+// bucket read as 128 and 64 bits two.
+struct Bucket {
+    uint32_t cnt[4], lo, hi, pad[2];
+};
+__device__ __forceinline__ Bucket load_bucket(const FmEntry *e)
 {
-    const FmEntry *e = F.occ + (i >> 5);
-    const int y = (int)(i & 31);
-    const uint4 c = __ldg(reinterpret_cast<const uint4 *>(e->cnt));
-    const uint64_t w = __ldg(&e->bwt);
-    const uint64_t m = (y ? (~0ull >> (64 - 2 * y)) : 0ull) & 0x5555555555555555ull;   // bit 2j, j < y
-    const uint64_t lo = w & m, hi = (w >> 1) & m;                                        // the two bits of base j
-    o[0] = c.x + (uint32_t)__popcll(m & ~lo & ~hi);
-    o[1] = c.y + (uint32_t)__popcll(lo & ~hi);
-    o[2] = c.z + (uint32_t)__popcll(hi & ~lo);
-    o[3] = c.w + (uint32_t)__popcll(lo & hi);
-    if (F.primary >= (int64_t)(i - y) && F.primary < (int64_t)i) --o[0];   // the $ row, stored as base 0
+    Bucket v;
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(v.cnt[0]), "=r"(v.cnt[1]), "=r"(v.cnt[2]), "=r"(v.cnt[3]), "=r"(v.lo), "=r"(v.hi), "=r"(v.pad[0]), "=r"(v.pad[1])
+        : "l"(e));
+    return v;
 }
 
-// The bi-interval of bP from that of P (Algorithm 2's backward extension).
-// A forward extension (Algorithm 3) is the same step: the bi-interval of Pc
-// is that of comp(c) revcomp(P) with the two intervals swapped.
-// [k', k'+s') holds the suffixes of [k, k+s) preceded by b.  revcomp(bP) =
-// revcomp(P) comp(b), whose interval inside [l, l+s) comes after the suffix
-// revcomp(P)$ (if any) and the extensions by bases smaller than comp(b), i.e.
-// after as many rows as P has occurrences preceded by the terminator or by a
-// base larger than b.
-__device__ __forceinline__ BiIv back_ext(const FmDev &F, const uint32_t C[5], BiIv v, int b)
+// What a lookup of O at row i gives for base b (Algorithm 1): row = C[b] + the
+// occurrences of b in BWT[0, i), and above = those of the bases larger than b
+// plus a constant (only differences of it are used).
+struct Occ {
+    uint32_t row, above;
+};
+__device__ __forceinline__ Occ occ_in(const FmDev &F, const Bucket &v, uint32_t i, uint32_t b)
 {
-    uint32_t ok[4], oe[4];
-    occ4(F, v.k, ok);
-    occ4(F, v.k + v.s, oe);
-    uint32_t above = 0;
-#pragma unroll
-    for (int c = 3; c > 0; --c)
-        if (c > b) above += oe[c] - ok[c];
-    const uint32_t sent = (F.primary >= (int64_t)v.k && F.primary < (int64_t)v.k + v.s) ? 1u : 0u;
-    uint32_t kb = ok[0], sb = oe[0] - ok[0];
-#pragma unroll
-    for (int c = 1; c < 4; ++c)
-        if (c == b) { kb = ok[c]; sb = oe[c] - ok[c]; }
-    return BiIv{C[b] + kb, v.l + sent + above, sb, v.e};
+    const uint32_t y = i & 31u;
+    const uint32_t m = (1u << y) - 1u;                                       // bases j < y
+    const uint32_t x = v.lo ^ (0u - (b & 1u)), z = v.hi ^ (0u - (b >> 1));   // both bits zero where base j is b
+    Occ o;
+    o.row = (b < 2 ? (b == 0 ? v.cnt[0] : v.cnt[1]) : (b == 2 ? v.cnt[2] : v.cnt[3])) + (uint32_t)__popc(~(x | z) & m);
+    if (b == 0 && F.primary - (i - y) < y) --o.row;                          // the $ row, stored as base 0
+    // larger than 0: either bit set; than 1: the high one; than 2: both
+    const uint32_t g = b == 0 ? (v.lo | v.hi) : b == 1 ? v.hi : b == 2 ? (v.lo & v.hi) : 0u;
+    const uint32_t zw = v.cnt[2] + v.cnt[3];
+    o.above = (b == 0 ? v.cnt[1] + zw : b == 1 ? zw : b == 2 ? v.cnt[3] : 0u) + (uint32_t)__popc(g & m);
+    return o;
 }
 
-// Base pos of the reads: 0..3, or 4 for an N.
-__device__ __forceinline__ int read_base(const SmemIn &R, int64_t pos)
+// The extension of the rows [a, a + s) by base b (Algorithm 2): the rows of bP
+// are [row, row + size); above = the occurrences among the s rows' preceding
+// bases of those larger than b.  Both ends of a small interval usually lie in
+// one bucket, which is then read once.
+struct Ext {
+    uint32_t row, size, above;
+};
+__device__ __forceinline__ Ext extend(const FmDev &F, uint32_t a, uint32_t s, uint32_t b)
 {
-    if (R.reads_n && ((__ldg(R.reads_n + (pos >> 3)) >> (pos & 7)) & 1)) return 4;
-    return (__ldg(R.reads + (pos >> 2)) >> (2 * (pos & 3))) & 3;
+    const uint32_t e = a + s;
+    const Bucket v0 = load_bucket(F.occ + (a >> 5));
+    Bucket v1 = v0;
+    if ((e >> 5) != (a >> 5)) v1 = load_bucket(F.occ + (e >> 5));
+    const Occ o0 = occ_in(F, v0, a, b), o1 = occ_in(F, v1, e, b);
+    return Ext{o0.row, o1.row - o0.row, o1.above - o0.above};
 }
+
+// C[c], the first row of base c (c = 4: past the last).
+__device__ __forceinline__ uint32_t first_row(const FmDev &F, int c)
+{
+    return c < 2 ? (c == 0 ? F.C[0] : F.C[1]) : c == 2 ? F.C[2] : c == 3 ? F.C[3] : F.C[4];
+}
+
+// A read of the batch: its packed bases (a read starts on a byte) and its base
+// offset, which addresses the N bitmap.
+struct ReadRef {
+    const uint8_t *q;
+    int64_t off;
+    __device__ __forceinline__ ReadRef() : q(nullptr), off(0) {}
+    __device__ __forceinline__ ReadRef(const SmemIn &R, int64_t o) : q(R.reads + (o >> 2)), off(o) {}
+    // Base pos: 0..3, or 4 for an N.
+    __device__ __forceinline__ int base(const SmemIn &R, int pos) const
+    {
+        if (R.reads_n && ((__ldg(R.reads_n + ((off + pos) >> 3)) >> ((off + pos) & 7)) & 1)) return 4;
+        return (__ldg(q + (pos >> 2)) >> (2 * (pos & 3))) & 3;
+    }
+};
 
 // All SMEMs of at least min_len bases of the reads t < t_end taken from the
-// counter *W.next (read ids[t], or t when ids is null), in increasing start
-// order.  Store mode: count[r], and the first kSmemKeep records at
-// scratch[r * kSmemKeep]; a read with more is finished by a write-mode launch.
-// Write mode: the records at out[first[r]].  A lane's list holds cap entries
-// at list[0], list[stride], ...; in store mode a read that needs more is
-// dropped (count -1, its id appended to ovf_list) and finished by a launch
-// with longer lists.
+// counter *W.next (read ids[t]).  Store mode: count[r], and the first kSmemKeep
+// matches at scratch[r * kSmemKeep], in the order they are found
+// (k_smem_gather sorts them); a read with more is finished by a write-mode
+// launch.  Write mode: the records at out[first[r]], in increasing start order.
+// A lane's list holds cap entries, enough for any read of the batch.
 //
 // The lane is a small state machine so that every pass of the main loop makes
-// exactly one bi-interval extension on every lane that has work (the memory
-// lookups of Algorithm 1 dominate; lanes of a warp run in step instead of
-// each following its own loop nest).  States between extensions:
+// exactly one extension on every lane that has work (the memory lookups of
+// Algorithm 1 dominate; lanes of a warp run in step instead of each following
+// its own loop nest).  States between extensions:
 //   kRead  take the next read;     kCall  start the search from x;
 //   kBack  forward pass over, start the backward pass;
 //   kEnd   the search from x is over;
-//   kFwd   pending: extend v forward by X[i];
-//   kBwd   pending: extend list[p] backward by X[j].
+//   kFwd   pending: extend the match forward by X[i];
+//   kBwd   pending: extend the list's p-th longest match backward by X[j].
+//
+// An extension of P by base b on the left (Algorithm 2) maps its rows [k, k +
+// s) to [C[b] + O(b, k), C[b] + O(b, k + s)).  A forward extension by c
+// (Algorithm 3) is the same step on revcomp(P)'s rows [l, l + s) with b = 3 -
+// c, and P's rows move up by as many as revcomp(P) has occurrences preceded by
+// the terminator or by a base larger than b (they sort before); a backward one
+// needs no more than the rows, as no forward extension follows.
 template <bool WRITE>
-__device__ void smem_lanes(const SmemIn &R, const FmDev &F, const uint32_t C[5], int min_len, int64_t t_end,
-                           const int32_t *ids, BiIv *list, int stride, int cap, const SmemWork &W)
+__device__ void smem_lanes(const SmemIn &R, const FmDev &F, int min_len, int64_t t_end, const int32_t *ids,
+                           BiIv *list, int cap, const SmemWork &W)
 {
     enum { kRead, kCall, kBack, kEnd, kFwd, kBwd };
     int state = kRead;
-    int64_t r = 0, base = 0, o = 0, n = 0, call0 = 0;
-    int L = 0, x = 0, i = 0, j = 0, p = 0, m = 0, mc = 0, next = 0, last = 0;
-    BiIv v{0, 0, 0, 0};
-    auto emit = [&](int start, int len, const BiIv &u) {
-        if (len < min_len) return;
-        bsw_smem_t sm;
-        sm.read_id = (int32_t)r;
-        sm.qbeg = start;
-        sm.len = len;
-        sm.reserved = 0;
-        sm.k = u.k;
-        sm.s = u.s;
-        if (WRITE) W.out[o + n] = sm;
-        else if (n < kSmemKeep) W.scratch[o + n] = sm;
+    int r = 0, n = 0, call0 = 0;
+    int64_t o = 0;
+    int L = 0, x = 0, i = 0, j = 0, p = 0, m = 0, mc = 0, top = 0, next = 0, last = 0;
+    uint32_t vk = 0, vl = 0, vs = 0, ls = 0;                            // the forward match; the last survivor's size
+    ReadRef read;
+    auto base_at = [&](int pos) { return read.base(R, pos); };
+    auto emit = [&](int start, int end, uint32_t k, uint32_t s) {
+        if (end - start < min_len) return;
+        if (WRITE) W.out[o + n] = bsw_smem_t{(int32_t)r, start, end - start, 0, (int64_t)k, (int64_t)s};
+        else if (n < kSmemKeep) W.scratch[o + n] = make_uint4((uint32_t)start, (uint32_t)(end - start), k, s);
         ++n;
     };
     for (;;) {
@@ -168,10 +204,10 @@ __device__ void smem_lanes(const SmemIn &R, const FmDev &F, const uint32_t C[5],
             if (state == kRead) {
                 const int64_t t = atomicAdd(W.next, 1u);
                 if (t >= t_end) return;
-                r = ids ? ids[t] : t;
+                r = ids[t];
                 L = R.read_len[r];
-                base = R.read_off[r];
-                o = WRITE ? W.first[r] : r * kSmemKeep;
+                read = ReadRef(R, R.read_off[r]);
+                o = WRITE ? W.first[r] : (int64_t)r * kSmemKeep;
                 n = 0;
                 x = 0;
                 state = kCall;
@@ -181,28 +217,27 @@ __device__ void smem_lanes(const SmemIn &R, const FmDev &F, const uint32_t C[5],
                     state = kRead;
                     continue;
                 }
-                const int c0 = read_base(R, base + x);
+                const int c0 = base_at(x);
                 if (c0 > 3) {                                           // no match starts at an N
                     ++x;
                     continue;
                 }
-                v = BiIv{C[c0], C[3 - c0], C[c0 + 1] - C[c0], 0};
+                vk = first_row(F, c0);
+                vl = first_row(F, 3 - c0);
+                vs = first_row(F, c0 + 1) - vk;
                 m = 0;
                 i = x + 1;
                 if (i < L) {
                     state = kFwd;
                 } else {
-                    v.e = L;
-                    list[(m++) * stride] = v;
+                    list[m++] = BiIv{vk, vs, L};
                     state = kBack;
                 }
             } else if (state == kBack) {
-                for (int a = 0, b = m - 1; a < b; ++a, --b) {          // longest first
-                    const BiIv u = list[a * stride];
-                    list[a * stride] = list[b * stride];
-                    list[b * stride] = u;
-                }
-                next = list[0].e;
+                // the list is in order of increasing length: the p-th longest
+                // is entry top - p, and survivors go back from the top down
+                top = m - 1;
+                next = list[top].e;
                 call0 = n;
                 last = INT_MAX;
                 j = x - 1;
@@ -211,58 +246,59 @@ __device__ void smem_lanes(const SmemIn &R, const FmDev &F, const uint32_t C[5],
                 if (j >= 0) {
                     state = kBwd;
                 } else {                                                // at the read start: the longest is an SMEM
-                    emit(0, list[0].e, list[0]);
+                    emit(0, next, list[top].k, list[top].s);
                     state = kEnd;
                 }
             } else {                                                    // kEnd
                 // this search emitted starts in decreasing order
-                bsw_smem_t *seg = WRITE ? W.out : W.scratch;
-                if (WRITE || n <= kSmemKeep)
+                if (WRITE)
                     for (int64_t a = o + call0, b = o + n - 1; a < b; ++a, --b) {
-                        const bsw_smem_t u = seg[a];
-                        seg[a] = seg[b];
-                        seg[b] = u;
+                        const bsw_smem_t u = W.out[a];
+                        W.out[a] = W.out[b];
+                        W.out[b] = u;
                     }
                 x = next;
                 state = kCall;
             }
         }
 
-        // one extension (Algorithm 2), the same code on every lane
+        // one extension, the same code on every lane
         const bool fwd = state == kFwd;
-        const BiIv u = fwd ? BiIv{v.l, v.k, v.s, 0} : list[p * stride];
-        const int cb = read_base(R, base + (fwd ? i : j));
-        BiIv w = back_ext(F, C, u, fwd ? 3 - (cb & 3) : cb & 3);
-        if (cb > 3) w.s = 0;                                        // an N extends nothing
+        uint32_t a = vl, s = vs;
+        if (!fwd) {
+            a = list[top - p].k;
+            s = list[top - p].s;
+        }
+        const int cb = base_at(fwd ? i : j);
+        const uint32_t b = (uint32_t)(fwd ? 3 - (cb & 3) : cb & 3);
+        const Ext u = extend(F, a, s, b);
+        const uint32_t s2 = cb > 3 ? 0u : u.size;                       // an N extends nothing
 
         if (fwd) {
-            w = BiIv{w.l, w.k, w.s, 0};
-            if (w.s != v.s) {                                       // X[x..i) is the longest with its count
-                if (m == cap) goto overflow;
-                v.e = i;
-                list[(m++) * stride] = v;
-                if (w.s == 0) {
+            if (s2 != vs) {                                             // X[x..i) is the longest with its count
+                list[m++] = BiIv{vk, vs, i};
+                if (s2 == 0) {
                     state = kBack;
                     continue;
                 }
             }
-            v = w;
-            if (++i == L) {                                         // the match reaches the read end
-                if (m == cap) goto overflow;
-                v.e = L;
-                list[(m++) * stride] = v;
+            vk += u.above + (F.primary - a < s ? 1u : 0u);
+            vl = u.row;
+            vs = s2;
+            if (++i == L) {                                             // the match reaches the read end
+                list[m++] = BiIv{vk, vs, L};
                 state = kBack;
             }
-            continue;
         } else {
-            if (w.s == 0) {
-                if (mc == 0 && j + 1 < last) {                      // no longer match survives: an SMEM
+            if (s2 == 0) {
+                if (mc == 0 && j + 1 < last) {                          // no longer match survives: an SMEM
                     last = j + 1;
-                    emit(last, u.e - last, u);
+                    emit(last, list[top - p].e, a, s);
                 }
-            } else if (mc == 0 || w.s != list[(mc - 1) * stride].s) {
-                w.e = u.e;
-                list[(mc++) * stride] = w;
+            } else if (mc == 0 || s2 != ls) {
+                list[top - mc] = BiIv{u.row, s2, list[top - p].e};
+                ls = s2;
+                ++mc;
             }
             if (++p == m) {
                 if (mc == 0) {
@@ -271,36 +307,212 @@ __device__ void smem_lanes(const SmemIn &R, const FmDev &F, const uint32_t C[5],
                     m = mc;
                     mc = 0;
                     p = 0;
-                    if (--j < 0) {                                  // at the read start
-                        emit(0, list[0].e, list[0]);
+                    if (--j < 0) {                                      // at the read start
+                        emit(0, list[top].e, list[top].k, list[top].s);
                         state = kEnd;
                     }
                 }
             }
-            continue;
         }
-    overflow:
-        if (!WRITE) {
-            W.count[r] = -1;
-            W.ovf_list[atomicAdd(W.ovf_n, 1u)] = (int32_t)r;
-        }
-        state = kRead;
     }
 }
 
-__device__ __forceinline__ void load_c(const FmDev &F, uint32_t C[5])
+// Store mode: counts and scratch records by atomics, as several lanes may work
+// on one read.  A read whose list does not fit is marked with kSmemOvf, which no
+// count reaches, and listed once.
+constexpr unsigned long long kSmemOvf = 1ull << 40;
+
+__device__ __forceinline__ void emit_match(const SmemWork &W, int min_len, int r, int start, int end, uint32_t k, uint32_t s)
 {
-#pragma unroll
-    for (int c = 0; c < 5; ++c) C[c] = (uint32_t)F.C[c];
+    if (end - start < min_len) return;
+    const unsigned long long n = atomicAdd(reinterpret_cast<unsigned long long *>(W.count + r), 1ull);
+    if (n < kSmemKeep) W.scratch[(int64_t)r * kSmemKeep + n] = make_uint4((uint32_t)start, (uint32_t)(end - start), k, s);
 }
 
-// Store mode over all reads with the lists in shared memory.
-__global__ void __launch_bounds__(kSmemThreads) k_smem_store(SmemIn R, FmDev F, int min_len, SmemWork W)
+__device__ __forceinline__ void overflow_read(const SmemWork &W, int r)
 {
-    extern __shared__ BiIv lists[];
-    uint32_t C[5];
-    load_c(F, C);
-    smem_lanes<false>(R, F, C, min_len, R.n_reads, nullptr, lists + threadIdx.x, blockDim.x, kListCap, W);
+    if (atomicAdd(reinterpret_cast<unsigned long long *>(W.count + r), kSmemOvf) < kSmemOvf)
+        W.ovf_list[atomicAdd(W.ovf_n, 1u)] = r;
+}
+
+// The starts of the searches of groups [g0, g0 + ng): a warp takes 32 reads, a lane one of
+// them, a base per step.  The longest match from the read's start is an SMEM;
+// the other starts go to the group's part of W.starts (start | lane << 16).
+__global__ void __launch_bounds__(kSmemThreads) k_smem_scan(SmemIn R, FmDev F, int min_len, SmemWork W, int64_t g0, int64_t ng)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    const int64_t g = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (g >= ng) return;
+    const int64_t r64 = (g0 + g) * 32 + lane;
+    const int r = (int)r64;
+    const bool mine = r64 < R.n_reads;
+    const int L = mine ? R.read_len[r] : 0;
+    ReadRef read;
+    if (mine) read = ReadRef(R, R.read_off[r]);
+    uint32_t *starts = W.starts + g * W.starts_cap;
+    uint32_t quad = 0;
+    int i = 0, x = -1, n = 0;                // the next base; the search's start (-1: none); starts noted
+    uint32_t vk = 0, vl = 0, vs = 0;         // the match X[x..i), its rows and those of its reverse complement
+    while (__any_sync(kAll, i < L)) {
+        if ((i & 3) == 0 && i < L) quad = __ldg(read.q + (i >> 2));       // four bases; their N bits come one by one
+        const int c = i >= L ? 4 : R.reads_n ? read.base(R, i) : (int)((quad >> (2 * (i & 3))) & 3u);
+        const uint32_t b = 3u - (uint32_t)(c & 3);
+        const Ext u = extend(F, vl, vs, b);
+        const uint32_t s2 = c < 4 ? u.size : 0u;
+        const bool ends = i < L && x >= 0 && s2 == 0 && vs > 0;
+        if (ends && x == 0) emit_match(W, min_len, r, 0, i, vk, vs);
+        const bool starts_here = i < L && (x < 0 || ends) && c < 4;     // no match starts at an N
+        if (starts_here) {
+            vk = first_row(F, c);
+            vl = first_row(F, 3 - c);
+            vs = first_row(F, c + 1) - vk;
+        } else {
+            vk += u.above + (F.primary - vl < vs ? 1u : 0u);
+            vl = u.row;
+            vs = s2;
+        }
+        const unsigned st = __ballot_sync(kAll, starts_here && i > 0);
+        if (starts_here && i > 0) {
+            const int at = n + __popc(st & below);
+            if (at < W.starts_cap) starts[at] = (uint32_t)i | ((uint32_t)lane << 16);
+            else overflow_read(W, r);
+        }
+        n += __popc(st);
+        if (starts_here) x = i;
+        else if (ends) x = -1;
+        if (i < L && ++i == L) {
+            if (x == 0) emit_match(W, min_len, r, 0, L, vk, vs);
+            vl = vs = 0;                                                  // done: look up row 0
+        }
+    }
+    if (lane == 0) W.n_starts[g] = (uint32_t)min(n, W.starts_cap);
+}
+// The searches from the noted starts: a warp works through the starts of
+// groups of 32 reads, its lanes taking the next one as they finish.  A lane's
+// matches lie in shared memory, 10 bytes each: rows and end (the rows of
+// revcomp(P), which the forward search needs, play no part once it is over).
+// A pass of the main loop makes one extension on every lane, forward or
+// backward; a forward one is a backward one of revcomp(P), see smem_lanes.
+// Bound by the lookups (random 32-byte reads, mostly L2 hits).  200 k reads of
+// 151 bp against a 32 Mbp text: k_smem_scan 0.29 ms and this kernel 1.12 ms, with
+// 25 and 18 of 32 lanes active; one kernel with a lane per read, lists of 16-byte
+// entries and two loads per bucket took 1.84 ms at 15 lanes.  24 matches a lane
+// and 7 blocks an SM run as fast as 28 and 6, 1% faster than 20 and 8.
+__global__ void __launch_bounds__(kSmemThreads) k_smem_store(SmemIn R, FmDev F, int min_len, SmemWork W, int64_t g0, int64_t ng)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    __shared__ uint2 ks[kListCap * kSmemThreads];
+    __shared__ uint16_t ends[kListCap * kSmemThreads];
+    const int lane = threadIdx.x & 31, me = threadIdx.x;
+    const unsigned below = (1u << lane) - 1u;
+    int64_t g = 0;                           // the warp's group of reads, its starts and the next of them
+    int nq = 0, head = 0;
+    bool left = true;                        // groups are left
+    int r = -1, L = 0, x = 0, i = 0, j = 0;  // the lane's read (-1: none), the search's start; the next base either way
+    ReadRef read;
+    bool fwd = true;
+    int c = 4, cpos = -1;                    // the base last read, and its position
+    int m = 0, p = 0, mc = 0, top = 0, last = 0;
+    uint32_t vk = 0, vl = 0, vs = 0, ls = 0; // the forward match; the last survivor's count
+    for (;;) {
+        if (head == nq && left) {
+            uint32_t t = 0;
+            if (lane == 0) t = atomicAdd(W.next, 1u);
+            g = (int64_t)__shfl_sync(kAll, t, 0);
+            left = g < ng;
+            nq = left ? (int)W.n_starts[g] : 0;
+            head = 0;
+        }
+        const unsigned want = __ballot_sync(kAll, r < 0);
+        if (want && head < nq) {
+            const int t = head + __popc(want & below);
+            if (r < 0 && t < nq) {
+                const uint32_t st = W.starts[g * W.starts_cap + t];
+                r = (int)((g0 + g) * 32 + (st >> 16));
+                x = (int)(st & 0xffffu);
+                read = ReadRef(R, R.read_off[r]);
+                L = R.read_len[r];
+                c = read.base(R, x);                                     // a base: no search starts at an N
+                cpos = x;
+                vk = first_row(F, c);
+                vl = first_row(F, 3 - c);
+                vs = first_row(F, c + 1) - vk;
+                i = x + 1;
+                m = 0;
+                fwd = true;
+            }
+            head = min(head + __popc(want), nq);
+        }
+        if (__ballot_sync(kAll, r >= 0) == 0) {
+            if (!left && head == nq) return;
+        } else if (r >= 0) {
+            const int pos = fwd ? i : j;
+            if (pos != cpos) {
+                c = pos < L ? read.base(R, pos) : 4;                     // the read's end stops a search as an N does
+                cpos = pos;
+            }
+            uint32_t a = vl, s = vs;
+            if (!fwd) {
+                const uint2 q = ks[(top - p) * kSmemThreads + me];
+                a = q.x;
+                s = q.y;
+            }
+            const uint32_t b = (uint32_t)(fwd ? 3 - (c & 3) : c & 3);
+            const Ext u = extend(F, a, s, b);
+            const uint32_t s2 = c < 4 ? u.size : 0u;
+            if (fwd) {
+                if (s2 != vs || i == L) {                                // X[x..i) is the longest with its count
+                    if (m < kListCap) {
+                        ks[m * kSmemThreads + me] = make_uint2(vk, vs);
+                        ends[m * kSmemThreads + me] = (uint16_t)i;
+                        ++m;
+                        if (s2 == 0) {                                   // the forward pass is over
+                            fwd = false;
+                            top = m - 1;
+                            p = mc = 0;
+                            j = x - 1;
+                            last = INT_MAX;
+                        }
+                    } else {
+                        overflow_read(W, r);
+                        r = -1;
+                    }
+                }
+                vk += u.above + (F.primary - a < s ? 1u : 0u);
+                vl = u.row;
+                vs = s2;
+                ++i;
+            } else {
+                // longest first: the list is in order of increasing length, the
+                // p-th longest is entry top - p, and survivors go back from the
+                // top down
+                if (s2 == 0) {
+                    if (mc == 0 && j + 1 < last) {                       // no longer match survives: an SMEM
+                        last = j + 1;
+                        emit_match(W, min_len, r, last, ends[(top - p) * kSmemThreads + me], a, s);
+                    }
+                } else if (mc == 0 || s2 != ls) {
+                    ks[(top - mc) * kSmemThreads + me] = make_uint2(u.row, s2);
+                    ends[(top - mc) * kSmemThreads + me] = ends[(top - p) * kSmemThreads + me];
+                    ls = s2;
+                    ++mc;
+                }
+                if (++p == m) {
+                    m = mc;
+                    p = mc = 0;
+                    if (m == 0) {
+                        r = -1;
+                    } else if (--j < 0) {                                // at the read start
+                        const uint2 v = ks[top * kSmemThreads + me];
+                        emit_match(W, min_len, r, 0, ends[top * kSmemThreads + me], v.x, v.y);
+                        r = -1;
+                    }
+                }
+            }
+        }
+    }
 }
 
 // The reads ids[0..n_ids) with lists in global memory, cap entries per lane
@@ -309,21 +521,26 @@ template <bool WRITE>
 __global__ void __launch_bounds__(256) k_smem_global(SmemIn R, FmDev F, int min_len, SmemWork W, const int32_t *ids,
                                                      int64_t n_ids, BiIv *lists, int cap)
 {
-    uint32_t C[5];
-    load_c(F, C);
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= n_ids) return;                     // at most n_ids lanes take reads: list slots g < n_ids
-    smem_lanes<WRITE>(R, F, C, min_len, n_ids, ids, lists + g * cap, 1, cap, W);
+    smem_lanes<WRITE>(R, F, min_len, n_ids, ids, lists + g * cap, cap, W);
 }
 
-// Records of the reads with at most kSmemKeep from the scratch to out[first[r]].
+// Records of the reads with at most kSmemKeep from the scratch to out[first[r]],
+// sorted by start (a read's SMEMs have distinct starts).
 __global__ void __launch_bounds__(256) k_smem_gather(int64_t n_reads, SmemWork W)
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n_reads; r += stride) {
-        const int64_t c = W.count[r];
+        const int c = (int)W.count[r];
         if (c > kSmemKeep) continue;
-        for (int64_t k = 0; k < c; ++k) W.out[W.first[r] + k] = W.scratch[r * kSmemKeep + k];
+        const uint4 *v = W.scratch + r * kSmemKeep;
+        for (int k = 0; k < c; ++k) {
+            const uint4 u = v[k];
+            int rank = 0;
+            for (int q = 0; q < c; ++q) rank += v[q].x < u.x;
+            W.out[W.first[r] + rank] = bsw_smem_t{(int32_t)r, (int32_t)u.x, (int32_t)u.y, 0, (int64_t)u.z, (int64_t)u.w};
+        }
     }
 }
 
@@ -335,16 +552,22 @@ int grid_for(int64_t n, int per_block, int sms, int per_sm)
 
 }  // namespace
 
-cudaError_t launch_smem_store(const SmemIn &R, const FmDev &F, int min_len, const SmemWork &W, cudaStream_t st, int sms)
+cudaError_t launch_smem_store(const SmemIn &R, const FmDev &F, int min_len, const SmemWork &W, int64_t chunk,
+                              cudaStream_t st, int sms)
 {
     if (R.n_reads <= 0) return cudaSuccess;
-    const size_t smem = sizeof(BiIv) * kListCap * kSmemThreads;
-    cudaError_t e = cudaFuncSetAttribute(k_smem_store, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaMemsetAsync(W.count, 0, sizeof(int64_t) * (size_t)R.n_reads, st);
     if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(W.next, 0, 4, st);
-    if (e != cudaSuccess) return e;
-    k_smem_store<<<grid_for(R.n_reads, kSmemThreads, sms, kSmemBlocksPerSm), kSmemThreads, smem, st>>>(R, F, min_len, W);
-    return cudaGetLastError();
+    const int64_t groups = (R.n_reads + 31) / 32;
+    constexpr int warps = kSmemThreads / 32;
+    for (int64_t g0 = 0; g0 < groups; g0 += chunk) {
+        const int64_t ng = groups - g0 < chunk ? groups - g0 : chunk;
+        if ((e = cudaMemsetAsync(W.next, 0, 4, st)) != cudaSuccess) return e;
+        k_smem_scan<<<(unsigned)((ng + warps - 1) / warps), kSmemThreads, 0, st>>>(R, F, min_len, W, g0, ng);
+        k_smem_store<<<grid_for(ng, warps, sms, kSmemBlocksPerSm), kSmemThreads, 0, st>>>(R, F, min_len, W, g0, ng);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_smem_global(bool write, const SmemIn &R, const FmDev &F, int min_len, const SmemWork &W,

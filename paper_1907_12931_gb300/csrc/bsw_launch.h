@@ -186,12 +186,13 @@ cudaError_t launch_filter(const DriverIn &D, int64_t n, bsw_aln_t *out, cudaStre
 
 // ----------------------------------------------------- FM-index and SMEMs
 
-// One bucket of the occurrence table: counts of each base in BWT[0, 32t)
-// and the bucket's 32 BWT bases, 2-bit packed (32 bytes, one DRAM sector).
+// One bucket of the occurrence table: for each base its first row plus its
+// occurrences in BWT[0, 32t), and the low and high bits of the bucket's 32 BWT
+// bases (32 bytes, one DRAM sector).
 struct FmEntry {
     uint32_t cnt[4];
-    uint64_t bwt;
-    uint64_t pad;
+    uint32_t lo, hi;
+    uint32_t pad[2];
 };
 
 // Host copy of one FM-index: n = text length + 1 BWT rows, the $ row, the
@@ -204,8 +205,8 @@ struct FmHost {
 
 struct FmDev {
     const FmEntry *occ;
-    int64_t n, primary;
-    int64_t C[5];
+    uint32_t primary;
+    uint32_t C[5];
 };
 
 // Reads of an SMEM search: packed 2-bit, read r at base offset read_off[r]
@@ -221,30 +222,38 @@ struct SmemIn {
 
 // The index of text[0..n) from its suffix array sa[0..n] (host).
 void fm_from_sa(const uint8_t *text, int64_t n, const int32_t *sa, FmHost &out);
-// end[r * lmax + i] = the end of the longest prefix of read r from i that
-// occurs in the text of Frev's reverse.
-// One bi-interval (Algorithm 2): [k, k + s) the suffix-array interval of a
-// match P in T, [l, l + s) that of revcomp(P), e the match's end in the read.
+// One match P of a read (Algorithm 2): [k, k + s) its suffix-array interval in
+// T, e its end in the read.
 struct BiIv {
-    uint32_t k, l, s;
+    uint32_t k, s;
     int32_t e;
 };
-constexpr int kSmemThreads = 128, kListCap = 24, kSmemBlocksPerSm = 4, kSmemKeep = 8;
+constexpr int kSmemThreads = 128, kListCap = 24, kSmemBlocksPerSm = 7, kSmemKeep = 8;
+// Search starts a group of 32 reads of at most lmax bases has room for.  Past a
+// sequencing error a search reaches about 13 bases, so twice that many fit.
+constexpr int smem_starts_cap(int lmax) { return 32 * (4 + lmax / 6); }
 
-// Buffers of one SMEM search.  Store mode: count[r] (-1 and r appended to
-// ovf_list[atomicAdd(ovf_n)] when the read's list exceeds kListCap) and up to
-// kSmemKeep records at scratch[r * kSmemKeep].  Write mode: records at
-// out[first[r]].  next: the launch's read counter (zeroed by the launchers).
+// Buffers of one SMEM search.  Store mode: count[r] (2^40 or more, and r once in
+// ovf_list[atomicAdd(ovf_n)], when a list of the read exceeds kListCap or its
+// starts the group's room) and up to
+// kSmemKeep matches {start, length, k, s} at scratch[r * kSmemKeep].  Write
+// mode: records at out[first[r]].  next: the launch's read counter (zeroed by the launchers).
 struct SmemWork {
     int64_t *count;
-    bsw_smem_t *scratch;
+    uint4 *scratch;
     const int64_t *first;
     bsw_smem_t *out;
     uint32_t *next;
     uint32_t *ovf_n;
     int32_t *ovf_list;
+    uint32_t *starts;        // [groups of 32 reads][starts_cap] search starts: start | lane << 16
+    uint32_t *n_starts;      // [groups]: the starts noted
+    int32_t starts_cap;
 };
-cudaError_t launch_smem_store(const SmemIn &R, const FmDev &F, int min_len, const SmemWork &W, cudaStream_t st, int sms);
+// W.starts and W.n_starts hold `chunk` groups; the reads are searched in as
+// many rounds as that takes.
+cudaError_t launch_smem_store(const SmemIn &R, const FmDev &F, int min_len, const SmemWork &W, int64_t chunk,
+                              cudaStream_t st, int sms);
 // The reads ids[0..n_ids) in store or write mode with lists in `lists` (cap
 // entries per lane, n_ids lanes at most).
 cudaError_t launch_smem_global(bool write, const SmemIn &R, const FmDev &F, int min_len, const SmemWork &W,

@@ -1,0 +1,85 @@
+"""The SMEM search's two kernels at their edges (needs a GPU).
+
+k_smem_scan takes groups of 32 reads and notes the searches' starts,
+k_smem_store works them off, in as many rounds as the budget's room for starts
+takes.  Cases: read counts around a group, empty and one-base reads, reads
+unrelated to the text (a start every dozen bases), and a budget that holds one
+group of starts at a time.
+"""
+import numpy as np
+import pytest
+
+from oracle import smem as oracle_smem
+from paper_1907_12931_gb300 import workload as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def bsw():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1907_12931_gb300 import bsw as _b
+    _b.lib()
+    return _b
+
+
+def make_reads(rng, ref, n, lmax):
+    out = []
+    for k in range(n):
+        ln = int(rng.choice([0, 1, 2, 40, lmax]))
+        p = int(rng.integers(0, len(ref) - lmax))
+        x = ref[p:p + ln].copy() if k % 3 else rng.integers(0, 4, ln).astype(np.uint8)
+        x[rng.random(ln) < 0.03] = 2
+        out.append(np.ascontiguousarray(3 - x[::-1]) if k & 1 else x)
+    return out
+
+
+def search(bsw, ctx, reads, min_len):
+    ln = np.array([len(x) for x in reads], np.int32)
+    off, total = W.layout(ln, 4)
+    codes = np.zeros(total, np.uint8)
+    for o, x in zip(off, reads):
+        codes[o:o + len(x)] = x
+    rec, first = ctx.smem(bsw.bsw_pack_2bit(codes), off, ln, min_len=min_len)
+    return [[tuple(int(rec[f][k]) for f in ("qbeg", "len", "k", "s")) for k in range(first[r], first[r + 1])]
+            for r in range(len(reads))]
+
+
+def expected(ref, reads, min_len):
+    return [[tuple(int(v) for v in rec) for rec in r] for r in oracle_smem.smems(ref, reads, min_len)]
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 64, 97])
+def test_group_edges(bsw, n):
+    rng = np.random.default_rng(n)
+    ref = rng.integers(0, 4, 1500).astype(np.uint8)
+    reads = make_reads(rng, ref, n, 130)
+    with bsw.Context(W.Params(), 1 << 30) as ctx:
+        ctx.fm_build(ref)
+        for min_len in (1, 7):
+            assert search(bsw, ctx, reads, min_len) == expected(ref, reads, min_len)
+
+
+def test_rounds_under_a_tight_budget(bsw):
+    """The smallest budgets that hold the reads and their records also hold the
+    search, group by group."""
+    rng = np.random.default_rng(8)
+    ref = rng.integers(0, 4, 2000).astype(np.uint8)
+    reads = make_reads(rng, ref, 300, 600)
+    want = expected(ref, reads, 12)
+    done = 0
+    for budget in range(200_000, 2_000_000, 25_000):
+        with bsw.Context(W.Params(), budget) as ctx:
+            ctx.fm_build(ref)
+            try:
+                got = search(bsw, ctx, reads, 12)
+            except bsw.BswError as e:
+                assert e.code == bsw.BSW_EBUDGET and done == 0
+                continue
+        assert got == want
+        done += 1
+        if done == 12:
+            break
+    assert done >= 3
