@@ -424,6 +424,7 @@ struct bsw_ctx {
     unsigned long long *h_cells = nullptr;
     Extents32 *h_ext = nullptr;
     DriverCheck *h_chk = nullptr;
+    SmemTotals *h_smem = nullptr;
 
     // execution plan (bsw_set_plan / bsw_autotune) and kernel timing
     Plan plan = default_plan();
@@ -1097,7 +1098,8 @@ int bsw_init(const bsw_scoring_t *sc, int32_t w, int32_t zdrop, int32_t end_bonu
     if (rc == BSW_OK && (cudaMallocHost(&c->h_status, 4) != cudaSuccess ||
                          cudaMallocHost(&c->h_cells, 8) != cudaSuccess ||
                          cudaMallocHost(&c->h_ext, sizeof(Extents32)) != cudaSuccess ||
-                         cudaMallocHost(&c->h_chk, sizeof(DriverCheck)) != cudaSuccess))
+                         cudaMallocHost(&c->h_chk, sizeof(DriverCheck)) != cudaSuccess ||
+                         cudaMallocHost(&c->h_smem, sizeof(SmemTotals)) != cudaSuccess))
         rc = BSW_ENOMEM;
     if (rc == BSW_OK && (cudaEventCreate(&c->tune_ev[0]) != cudaSuccess || cudaEventCreate(&c->tune_ev[1]) != cudaSuccess))
         rc = BSW_ECUDA;
@@ -1815,21 +1817,28 @@ int bsw_smem_n(bsw_ctx_t *ctx, int64_t n_reads, const uint8_t *reads, const uint
         *n_out = 0;
         if (first) first[0] = 0;
         if (n_reads == 0) return BSW_OK;
-        int64_t read_bytes = 0;
-        int lmax = 0;
+        // branch-free, so that the compiler vectorises it (200 k reads: 175 us with
+        // an early return per read)
+        int64_t bases_end = 0;
+        int32_t lmax = 0, bad = 0;
         for (int64_t r = 0; r < n_reads; ++r) {
-            if (read_off[r] < 0 || (read_off[r] & 3) || read_len[r] < 0 || read_len[r] > kLongMax) return BSW_EINVAL;
-            read_bytes = std::max(read_bytes, (read_off[r] + read_len[r] + 3) / 4);
-            lmax = std::max(lmax, (int)read_len[r]);
+            const int64_t off = read_off[r];
+            const int32_t len = read_len[r];
+            bad |= (int32_t)(off < 0) | (int32_t)(off & 3) | (int32_t)(len < 0) | (int32_t)(len > kLongMax);
+            bases_end = std::max(bases_end, (int64_t)((uint64_t)off + (uint64_t)(int64_t)len));
+            lmax = std::max(lmax, len);
         }
+        if (bad) return BSW_EINVAL;
+        const int64_t read_bytes = (bases_end + 3) / 4;
         size_t o = 0;
         auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes, 256); return r; };
         const int64_t groups = (n_reads + 31) / 32;
         const int starts_cap = smem_starts_cap(lmax);
         const size_t o_reads = take((size_t)read_bytes), o_roff = take(8 * (size_t)n_reads),
                      o_rlen = take(4 * (size_t)n_reads), o_cnt = take(8 * (size_t)n_reads),
-                     o_first = take(8 * (size_t)n_reads), o_ids = take(4 * (size_t)n_reads), o_nids = take(4),
-                     o_next = take(4), o_keep = take(sizeof(uint4) * kSmemKeep * (size_t)n_reads),
+                     o_first = take(8 * ((size_t)n_reads + 1)), o_ids = take(4 * (size_t)n_reads),
+                     o_many = take(4 * (size_t)n_reads), o_tot = take(sizeof(SmemTotals)),
+                     o_tile = take(8 * (size_t)smem_tiles(n_reads)), o_next = take(4), o_keep = take(sizeof(uint4) * kSmemKeep * (size_t)n_reads),
                      o_rn = take(reads_n ? (size_t)((read_bytes + 1) / 2) : 0),
                      o_out = take(sizeof(bsw_smem_t) * (size_t)std::max<int64_t>(out_cap, 1));
         // the search starts of as many groups at a time as the budget holds
@@ -1847,64 +1856,58 @@ int bsw_smem_n(bsw_ctx_t *ctx, int64_t n_reads, const uint8_t *reads, const uint
         cudaError_t e;
         if ((e = cudaMemcpyAsync(d + o_reads, reads, (size_t)read_bytes, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
             (e = cudaMemcpyAsync(d + o_roff, read_off, 8 * (size_t)n_reads, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-            (e = cudaMemcpyAsync(d + o_rlen, read_len, 4 * (size_t)n_reads, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-            (e = cudaMemsetAsync(d + o_nids, 0, 4, st)) != cudaSuccess)
+            (e = cudaMemcpyAsync(d + o_rlen, read_len, 4 * (size_t)n_reads, cudaMemcpyHostToDevice, st)) != cudaSuccess)
             return cuda_rc(e);
         if (reads_n && read_bytes &&
             (e = cudaMemcpyAsync(d + o_rn, reads_n, (size_t)((read_bytes + 1) / 2), cudaMemcpyHostToDevice, st)) != cudaSuccess)
             return cuda_rc(e);
         const SmemIn R{d + o_reads, (const int64_t *)(d + o_roff), (const int32_t *)(d + o_rlen), n_reads, lmax,
                        reads_n ? d + o_rn : nullptr};
-        int32_t *ids = (int32_t *)(d + o_ids);
-        uint32_t *nids = (uint32_t *)(d + o_nids);
-        int64_t *dfirst = (int64_t *)(d + o_first);
-        const SmemWork W{(int64_t *)(d + o_cnt), (uint4 *)(d + o_keep), dfirst, (bsw_smem_t *)(d + o_out),
-                         (uint32_t *)(d + o_next), nids, ids, (uint32_t *)(d + o_starts),
-                         (uint32_t *)(d + o_nst), starts_cap};
+        const SmemWork W{(int64_t *)(d + o_cnt), (uint4 *)(d + o_keep), (int64_t *)(d + o_first), (bsw_smem_t *)(d + o_out),
+                         (uint32_t *)(d + o_next), (SmemTotals *)(d + o_tot), (int32_t *)(d + o_ids), (int32_t *)(d + o_many),
+                         (int64_t *)(d + o_tile), (uint32_t *)(d + o_starts), (uint32_t *)(d + o_nst), starts_cap};
         auto global_lists = [&](int64_t n_ids, BiIv **lists) -> int {      // lmax + 1 entries hold any list
             const int r2 = ctx->smemscratch.reserve(sizeof(BiIv) * (size_t)n_ids * (size_t)(lmax + 1), ctx->budget);
             *lists = (BiIv *)ctx->smemscratch.p;
             return r2;
         };
 
-        // One search pass: counts, and the records of reads with few; reads whose
-        // lists overflow shared memory are searched with lists in global memory.
-        if ((e = launch_smem_store(R, ctx->fm_t, min_len, W, chunk, st, ctx->sms)) != cudaSuccess ||
-            (e = cudaMemcpyAsync(ctx->h_status, nids, 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-            (e = cudaStreamSynchronize(st)) != cudaSuccess)
-            return cuda_rc(e);
-        const int64_t n_ovf = *ctx->h_status;
+        // One search pass: counts, the records of reads with few, and the records'
+        // positions; reads whose lists overflow shared memory are searched with
+        // lists in global memory, which changes the counts.
+        auto positions = [&]() -> int {
+            cudaError_t pe;
+            if ((pe = launch_smem_first(n_reads, W, st)) != cudaSuccess ||
+                (pe = cudaMemcpyAsync(ctx->h_smem, W.totals, sizeof(SmemTotals), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
+                (pe = cudaStreamSynchronize(st)) != cudaSuccess)
+                return cuda_rc(pe);
+            return BSW_OK;
+        };
+        if ((e = launch_smem_store(R, ctx->fm_t, min_len, W, chunk, st, ctx->sms)) != cudaSuccess) return cuda_rc(e);
+        if ((rc = positions()) != BSW_OK) return rc;
+        const int64_t n_ovf = ctx->h_smem->overflows;
         if (n_ovf > 0) {
             BiIv *lists = nullptr;
             if ((rc = global_lists(n_ovf, &lists)) != BSW_OK) return rc;
-            if ((e = launch_smem_global(false, R, ctx->fm_t, min_len, W, ids, n_ovf, lists, lmax + 1, st, ctx->sms)) !=
+            if ((e = launch_smem_global(false, R, ctx->fm_t, min_len, W, W.ovf_list, n_ovf, lists, lmax + 1, st, ctx->sms)) !=
                 cudaSuccess)
                 return cuda_rc(e);
+            if ((rc = positions()) != BSW_OK) return rc;
         }
-        std::vector<int64_t> hc((size_t)n_reads), hf((size_t)n_reads + 1);
-        if ((e = cudaMemcpyAsync(hc.data(), W.count, 8 * (size_t)n_reads, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-            (e = cudaStreamSynchronize(st)) != cudaSuccess)
-            return cuda_rc(e);
-        hf[0] = 0;
-        std::vector<int32_t> many;                                        // reads with more records than were kept
-        for (int64_t r = 0; r < n_reads; ++r) {
-            hf[(size_t)r + 1] = hf[(size_t)r] + hc[(size_t)r];
-            if (hc[(size_t)r] > kSmemKeep) many.push_back((int32_t)r);
-        }
-        const int64_t total = hf[(size_t)n_reads];
+        const int64_t total = ctx->h_smem->records, n_many = ctx->h_smem->many;
         *n_out = total;
-        if (first) std::memcpy(first, hf.data(), 8 * ((size_t)n_reads + 1));
-        if (total > out_cap) return BSW_EBUDGET;
-        if (total == 0) return BSW_OK;
-        if ((e = cudaMemcpyAsync(dfirst, hf.data(), 8 * (size_t)n_reads, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-            (e = launch_smem_gather(n_reads, W, st, ctx->sms)) != cudaSuccess)
+        if (first && (e = cudaMemcpyAsync(first, W.first, 8 * ((size_t)n_reads + 1), cudaMemcpyDeviceToHost, st)) != cudaSuccess)
             return cuda_rc(e);
-        if (!many.empty()) {
+        if (total == 0 || total > out_cap) {
+            if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_rc(e);
+            return total == 0 ? BSW_OK : BSW_EBUDGET;
+        }
+        if ((e = launch_smem_gather(n_reads, W, st, ctx->sms)) != cudaSuccess) return cuda_rc(e);
+        if (n_many > 0) {
             BiIv *lists = nullptr;
-            if ((rc = global_lists((int64_t)many.size(), &lists)) != BSW_OK) return rc;
-            if ((e = cudaMemcpyAsync(ids, many.data(), 4 * many.size(), cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-                (e = launch_smem_global(true, R, ctx->fm_t, min_len, W, ids, (int64_t)many.size(), lists, lmax + 1, st,
-                                        ctx->sms)) != cudaSuccess)
+            if ((rc = global_lists(n_many, &lists)) != BSW_OK) return rc;
+            if ((e = launch_smem_global(true, R, ctx->fm_t, min_len, W, W.many, n_many, lists, lmax + 1, st, ctx->sms)) !=
+                cudaSuccess)
                 return cuda_rc(e);
         }
         if ((e = cudaMemcpyAsync(out, W.out, sizeof(bsw_smem_t) * (size_t)total, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
@@ -1948,6 +1951,7 @@ void bsw_destroy(bsw_ctx_t *ctx)
     if (ctx->h_cells) cudaFreeHost(ctx->h_cells);
     if (ctx->h_ext) cudaFreeHost(ctx->h_ext);
     if (ctx->h_chk) cudaFreeHost(ctx->h_chk);
+    if (ctx->h_smem) cudaFreeHost(ctx->h_smem);
     delete ctx;
 }
 

@@ -29,8 +29,8 @@
 // start per lane and does its forward and backward pass.  A read with more than
 // kListCap matches in one list is finished by a launch with lists in global
 // memory (k_smem_global), where a lane does a whole read.  One pass keeps up to
-// kSmemKeep records per read in a scratch buffer; after the host's prefix sum a
-// gather sorts them into place, and the rare reads with more are searched
+// kSmemKeep records per read in a scratch buffer; after a prefix sum of the
+// counts a gather sorts them into place, and the rare reads with more are searched
 // again, writing in place.
 #include <cuda_runtime.h>
 #include <climits>
@@ -332,7 +332,7 @@ __device__ __forceinline__ void emit_match(const SmemWork &W, int min_len, int r
 __device__ __forceinline__ void overflow_read(const SmemWork &W, int r)
 {
     if (atomicAdd(reinterpret_cast<unsigned long long *>(W.count + r), kSmemOvf) < kSmemOvf)
-        W.ovf_list[atomicAdd(W.ovf_n, 1u)] = r;
+        W.ovf_list[atomicAdd(&W.totals->overflows, 1u)] = r;
 }
 
 // The starts of the searches of groups [g0, g0 + ng): a warp takes 32 reads, a lane one of
@@ -526,6 +526,70 @@ __global__ void __launch_bounds__(256) k_smem_global(SmemIn R, FmDev F, int min_
     smem_lanes<WRITE>(R, F, min_len, n_ids, ids, lists + g * cap, cap, W);
 }
 
+// first[r] = the records before read r, first[n] = their number: sums of tiles of
+// kFirstTile reads, then each tile's prefix.  The reads with more records than
+// were kept are listed on the way.
+constexpr int kFirstThreads = 256, kFirstPer = 8, kFirstTile = kFirstThreads * kFirstPer;
+
+__device__ __forceinline__ int64_t block_sum(int64_t v)
+{
+    __shared__ int64_t w[kFirstThreads / 32];
+    for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+    if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = v;
+    __syncthreads();
+    int64_t t = 0;
+    for (int k = 0; k < kFirstThreads / 32; ++k) t += w[k];
+    __syncthreads();
+    return t;
+}
+
+__global__ void __launch_bounds__(kFirstThreads) k_smem_sums(int64_t n_reads, SmemWork W)
+{
+    int64_t v = 0;
+    for (int u = 0; u < kFirstPer; ++u) {
+        const int64_t r = (int64_t)blockIdx.x * kFirstTile + u * kFirstThreads + threadIdx.x;
+        const int64_t c = r < n_reads ? W.count[r] : 0;
+        if (c > kSmemKeep) W.many[atomicAdd(&W.totals->many, 1u)] = (int32_t)r;
+        v += c;
+    }
+    v = block_sum(v);
+    if (threadIdx.x == 0) W.tile_sum[blockIdx.x] = v;
+}
+
+__global__ void __launch_bounds__(kFirstThreads) k_smem_first(int64_t n_reads, SmemWork W)
+{
+    __shared__ int64_t warp_sum[kFirstThreads / 32];
+    int64_t before = 0;
+    for (int64_t b = threadIdx.x; b < blockIdx.x; b += kFirstThreads) before += W.tile_sum[b];
+    before = block_sum(before);
+    const int64_t r0 = (int64_t)blockIdx.x * kFirstTile + (int64_t)threadIdx.x * kFirstPer;
+    int64_t c[kFirstPer], sum = 0;
+#pragma unroll
+    for (int u = 0; u < kFirstPer; ++u) {
+        c[u] = r0 + u < n_reads ? W.count[r0 + u] : 0;
+        sum += c[u];
+    }
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int64_t x = sum;
+    for (int d = 1; d < 32; d <<= 1) {
+        const int64_t y = __shfl_up_sync(0xffffffffu, x, d);
+        if (lane >= d) x += y;
+    }
+    if (lane == 31) warp_sum[wid] = x;
+    __syncthreads();
+    int64_t at = before + x - sum;
+    for (int k = 0; k < wid; ++k) at += warp_sum[k];
+#pragma unroll
+    for (int u = 0; u < kFirstPer; ++u) {
+        if (r0 + u < n_reads) W.first[r0 + u] = at;
+        at += c[u];
+        if (r0 + u == n_reads - 1) {
+            W.first[n_reads] = at;
+            W.totals->records = at;
+        }
+    }
+}
+
 // Records of the reads with at most kSmemKeep from the scratch to out[first[r]],
 // sorted by start (a read's SMEMs have distinct starts).
 __global__ void __launch_bounds__(256) k_smem_gather(int64_t n_reads, SmemWork W)
@@ -552,12 +616,15 @@ int grid_for(int64_t n, int per_block, int sms, int per_sm)
 
 }  // namespace
 
+int64_t smem_tiles(int64_t n_reads) { return (n_reads + kFirstTile - 1) / kFirstTile; }
+
 cudaError_t launch_smem_store(const SmemIn &R, const FmDev &F, int min_len, const SmemWork &W, int64_t chunk,
                               cudaStream_t st, int sms)
 {
     if (R.n_reads <= 0) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(W.count, 0, sizeof(int64_t) * (size_t)R.n_reads, st);
     if (e != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(W.totals, 0, sizeof(SmemTotals), st)) != cudaSuccess) return e;
     const int64_t groups = (R.n_reads + 31) / 32;
     constexpr int warps = kSmemThreads / 32;
     for (int64_t g0 = 0; g0 < groups; g0 += chunk) {
@@ -579,6 +646,16 @@ cudaError_t launch_smem_global(bool write, const SmemIn &R, const FmDev &F, int 
     const int blocks = grid_for(n_ids, 256, sms, 8);
     if (write) k_smem_global<true><<<blocks, 256, 0, st>>>(R, F, min_len, W, ids, n_ids, lists, cap);
     else k_smem_global<false><<<blocks, 256, 0, st>>>(R, F, min_len, W, ids, n_ids, lists, cap);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_smem_first(int64_t n_reads, const SmemWork &W, cudaStream_t st)
+{
+    cudaError_t e = cudaMemsetAsync(&W.totals->many, 0, sizeof(uint32_t), st);
+    if (e != cudaSuccess) return e;
+    const unsigned tiles = (unsigned)smem_tiles(n_reads);
+    k_smem_sums<<<tiles, kFirstThreads, 0, st>>>(n_reads, W);
+    k_smem_first<<<tiles, kFirstThreads, 0, st>>>(n_reads, W);
     return cudaGetLastError();
 }
 

@@ -233,19 +233,27 @@ constexpr int kSmemThreads = 128, kListCap = 24, kSmemBlocksPerSm = 7, kSmemKeep
 // sequencing error a search reaches about 13 bases, so twice that many fit.
 constexpr int smem_starts_cap(int lmax) { return 32 * (4 + lmax / 6); }
 
+// What the host reads back of a search.
+struct SmemTotals {
+    uint32_t overflows, many;
+    int64_t records;
+};
+
 // Buffers of one SMEM search.  Store mode: count[r] (2^40 or more, and r once in
-// ovf_list[atomicAdd(ovf_n)], when a list of the read exceeds kListCap or its
+// ovf_list[totals->overflows++], when a list of the read exceeds kListCap or its
 // starts the group's room) and up to
 // kSmemKeep matches {start, length, k, s} at scratch[r * kSmemKeep].  Write
 // mode: records at out[first[r]].  next: the launch's read counter (zeroed by the launchers).
 struct SmemWork {
     int64_t *count;
     uint4 *scratch;
-    const int64_t *first;
+    int64_t *first;          // [n_reads + 1]
     bsw_smem_t *out;
     uint32_t *next;
-    uint32_t *ovf_n;
+    SmemTotals *totals;
     int32_t *ovf_list;
+    int32_t *many;           // reads with more than kSmemKeep records (totals->many)
+    int64_t *tile_sum;       // [smem_tiles(n_reads)]
     uint32_t *starts;        // [groups of 32 reads][starts_cap] search starts: start | lane << 16
     uint32_t *n_starts;      // [groups]: the starts noted
     int32_t starts_cap;
@@ -258,6 +266,10 @@ cudaError_t launch_smem_store(const SmemIn &R, const FmDev &F, int min_len, cons
 // entries per lane, n_ids lanes at most).
 cudaError_t launch_smem_global(bool write, const SmemIn &R, const FmDev &F, int min_len, const SmemWork &W,
                                const int32_t *ids, int64_t n_ids, BiIv *lists, int cap, cudaStream_t st, int sms);
+// first[] from the counts, the reads with more than kSmemKeep records, and the
+// number of records (totals).
+int64_t smem_tiles(int64_t n_reads);
+cudaError_t launch_smem_first(int64_t n_reads, const SmemWork &W, cudaStream_t st);
 // Records of reads with count <= kSmemKeep from the scratch to out[first[r]].
 cudaError_t launch_smem_gather(int64_t n_reads, const SmemWork &W, cudaStream_t st, int sms);
 
