@@ -334,7 +334,9 @@ int bsw_extend_batch_noalloc(const bsw_scoring_t *sc, int32_t w, int32_t zdrop, 
  * Execution plan of the batched path: which kernel runs which pairs.  The
  * paper fixes these choices for 512-bit vectors (Section V-C: sort by length,
  * 8-bit lanes first, 16-bit re-run); here they are parameters.  Every plan
- * computes the same results; plans differ only in speed.
+ * computes the same results; plans differ only in speed.  A batch of up to
+ * 12288 pairs runs the queries of the per-thread classes one per warp instead,
+ * unless packed is 1, lanes are forced or kernel times are asked for.
  *
  *   short_max    queries of up to short_max bases run one pair per thread (the
  *                per-thread length classes); longer ones one pair per warp.

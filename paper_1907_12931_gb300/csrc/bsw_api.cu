@@ -499,13 +499,13 @@ bool same_batch(const bsw_batch_t &a, const bsw_batch_t &b)
 // Enqueue one launch of a device-resident batch on the lane's streams (S.main
 // may be replaced by the caller's stream).  Zeroes cells/status first.
 cudaError_t enqueue_launch(bsw_ctx *c, Lane &lane, const Streams &S, const Batch &B, Work W, uint32_t flags,
-                           bool reset_status, const Plan &L, ClassTimer *T = nullptr)
+                           bool reset_status, const Plan &L, ClassTimer *T = nullptr, bool per_class = false)
 {
     cudaError_t e;
     Params P = c->P;
     P.flags = flags;
     const bool plain = (flags & (BSW_PLAIN_KERNEL | BSW_PLAIN_GLOBAL)) != 0;
-    c->last_launches = plain ? plain_launches(P, L, flags) : batched_launches(L, flags);
+    c->last_launches = plain ? plain_launches(P, L, flags) : batched_launches(B.n, flags, L, per_class);
     if (lane.work_dirty) {
         if ((e = cudaMemsetAsync(W.hist, 0, 4 * kNumBins, S.main)) != cudaSuccess) return e;
         lane.work_dirty = false;
@@ -513,7 +513,7 @@ cudaError_t enqueue_launch(bsw_ctx *c, Lane &lane, const Streams &S, const Batch
     if ((e = cudaMemsetAsync(W.cells, 0, 8, S.main)) != cudaSuccess) return e;
     if (reset_status && (e = cudaMemsetAsync(W.status, 0, 4, S.main)) != cudaSuccess) return e;
     if (fault_hit(BSW_FAULT_LAUNCH)) return cudaErrorLaunchFailure;
-    return plain ? launch_plain(B, P, W, S.main, c->sms, L) : launch_batched(B, P, W, S, c->sms, L, T);
+    return plain ? launch_plain(B, P, W, S.main, c->sms, L) : launch_batched(B, P, W, S, c->sms, L, T, per_class);
 }
 
 // Timing events for BSW_TIME_KERNELS (created on first use); nullptr when the
@@ -1391,7 +1391,7 @@ int bsw_autotune(bsw_ctx_t *ctx, const bsw_batch_t *b, int64_t sample_pairs, int
             for (int r = 0; r <= reps; ++r) {
                 cudaError_t e;
                 if ((e = cudaEventRecord(ctx->tune_ev[0], lane.S.main)) != cudaSuccess) return cuda_rc(e);
-                if ((e = enqueue_launch(ctx, lane, lane.S, B, W, 0u, true, L)) != cudaSuccess) {
+                if ((e = enqueue_launch(ctx, lane, lane.S, B, W, 0u, true, L, nullptr, true)) != cudaSuccess) {
                     lane.work_dirty = true;
                     return cuda_rc(e);
                 }

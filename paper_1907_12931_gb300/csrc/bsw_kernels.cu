@@ -2496,6 +2496,7 @@ constexpr int64_t kSpreadPairs = 393216;
 constexpr int kForkOrder[kNumClass] = {kClsCTA, 0, 1, 2, 3, 4, 5, 6, 7, kClsW16, kClsW32, 8, 9, 10, 11};
 constexpr int kClassStreamSmall[kNumClass] = {0, 1, 2, 3, 4, 5, 6, 7, 0, 1, 2, 3, 3, 5, 6};
 constexpr int kClassStreamLarge[kNumClass] = {0, 0, 1, 1, 2, 2, 3, 3, 0, 1, 2, 3, 3, 2, 2};
+constexpr int kClassStreamOne[kNumClass] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 1, 2, 3};   // classes 0-11 in one kernel
 
 // Whether class c can hold pairs under the plan and the batch flags (classes
 // that cannot are not launched).
@@ -2550,10 +2551,24 @@ cudaError_t launch_extents(const PairMeta &M, int64_t n, const Params &P, Extent
 
 bool packed_scoring_ok(const Params &P) { return inter2_scoring_ok(P); }
 
-int batched_launches(const Plan &L, uint32_t flags)
+// Up to this many pairs the short queries run one per warp.  The per-thread
+// kernels' time hardly depends on the number of pairs below some 20 k, that of
+// k_short grows with it: the two meet at about 12 k pairs of 1-130 base queries
+// (446 against 457 us), and past 16 k pairs of reads (151 bp: 320 against 403 us
+// at 16 k, 250 bp: 525 against 613; at 24 k 461 against 413 and 765 against 614).
+constexpr int64_t kShortPairs = 12288;
+
+bool short_path(int64_t n, uint32_t flags, const Plan &L, bool per_class)
 {
-    int k = 3;   // classify, scan, scatter
-    for (int c = 0; c <= kNumClass; ++c) k += class_live(c, L, flags) ? 1 : 0;
+    return n <= kShortPairs && !per_class && !L.packed &&
+           !(flags & (BSW_FORCE_I8 | BSW_FORCE_I16 | BSW_FORCE_I32 | BSW_PACKED_PAIRS | BSW_TIME_KERNELS));
+}
+
+int batched_launches(int64_t n, uint32_t flags, const Plan &L, bool per_class)
+{
+    const bool one = short_path(n, flags, L, per_class);
+    int k = one ? 4 : 3;   // classify, scan, scatter; the one kernel of the short queries
+    for (int c = one ? kClsCTA : 0; c <= kNumClass; ++c) k += class_live(c, L, flags) ? 1 : 0;
     return k;
 }
 
@@ -2597,7 +2612,7 @@ cudaError_t prepare_kernels(int sms)
 int warp_slots_needed(int sms) { return sms * kWarpBlocksPerSM * (kWarpKernelThreads / 32); }
 
 cudaError_t launch_batched(const Batch &B, const Params &P0, const Work &W, const Streams &S, int sms, const Plan &L,
-                           ClassTimer *T)
+                           ClassTimer *T, bool per_class)
 {
     cudaError_t e;
     if (B.n <= 0) return cudaSuccess;
@@ -2607,20 +2622,23 @@ cudaError_t launch_batched(const Batch &B, const Params &P0, const Work &W, cons
     // Fork: classes run concurrently on the side streams so that one class's
     // tail overlaps the next class's start.
     if ((e = cudaEventRecord(S.fork, S.main)) != cudaSuccess) return e;
-    for (int k = 0; k < kSideStreams; ++k)
+    const bool one = W.rec && short_path(B.n, P.flags, L, per_class);
+    const int *side = one ? kClassStreamOne : B.n <= kSpreadPairs ? kClassStreamSmall : kClassStreamLarge;
+    const int sides = one || B.n > kSpreadPairs ? 4 : kSideStreams;
+    for (int k = 0; k < sides; ++k)
         if ((e = cudaStreamWaitEvent(S.side[k], S.fork, 0)) != cudaSuccess) return e;
     const int wblocks = sms * kWarpBlocksPerSM;
-    const int *side = B.n <= kSpreadPairs ? kClassStreamSmall : kClassStreamLarge;
+    if (one && (e = launch_short(B, P, W, 0, kClsCTA, S.side[0], sms)) != cudaSuccess) return e;
     // The two-columns warp kernel runs after the other classes: it leaves a
     // quarter of each SM's block slots free (3 blocks of its 4, so the
     // longest pairs get a twelfth of an SM, not a sixteenth), and kernels of
     // other classes in them would take issue slots from those pairs.
     const bool x2_after = L.warp_x2 && x2_usable(P) && x2_ring_log2(P) > 0;
     for (int c : kForkOrder)
-        if (class_live(c, L, P.flags) && !(x2_after && c == kClsW16) &&
+        if (class_live(c, L, P.flags) && !(x2_after && c == kClsW16) && !(one && c < kClsCTA) &&
             (e = launch_class(c, B, P, W, S.side[side[c]], sms, wblocks, L, T)) != cudaSuccess)
             return e;
-    for (int k = 0; k < kSideStreams; ++k) {
+    for (int k = 0; k < sides; ++k) {
         if ((e = cudaEventRecord(S.join[k], S.side[k])) != cudaSuccess) return e;
         if ((e = cudaStreamWaitEvent(S.main, S.join[k], 0)) != cudaSuccess) return e;
     }

@@ -69,8 +69,16 @@ cudaError_t launch_plain_x2(const Batch &B, const Params &P, const Work &W, cuda
 // Whether the scoring lets the packed two-pairs-per-thread kernel run.
 bool packed_scoring_ok(const Params &P);
 
-// Kernels one launch_batched call makes under the plan and batch flags.
-int batched_launches(const Plan &L, uint32_t flags);
+// Whether a batch of n pairs is small enough for its short queries (classes
+// 0-11) to run one pair per warp with the row in registers (bsw_short.cu)
+// instead of one per thread.  per_class: the caller wants the plan's own
+// kernels (to time them).
+bool short_path(int64_t n, uint32_t flags, const Plan &L, bool per_class);
+cudaError_t launch_short(const Batch &B, const Params &P, const Work &W, int c0, int c1, cudaStream_t st, int sms);
+
+// Kernels one launch_batched call makes for n pairs under the plan and batch
+// flags.
+int batched_launches(int64_t n, uint32_t flags, const Plan &L, bool per_class);
 
 // Optional CUDA events around each class kernel (timing-enabled events,
 // recorded on the stream the kernel is launched on).
@@ -89,9 +97,10 @@ int warp_slots_needed(int sms);
 // Length-bucketed batched path: classify + counting sort + per-class
 // persistent kernels (forked over the side streams) + 32-bit re-run.
 // W.hist must be zero on entry (k_scan leaves it zero); W.cells and W.status
-// accumulate.  T (nullable) records each launched class kernel's events.
+// accumulate.  T (nullable) records each launched class kernel's events;
+// per_class as for short_path.
 cudaError_t launch_batched(const Batch &B, const Params &P, const Work &W, const Streams &S, int sms, const Plan &L,
-                           ClassTimer *T = nullptr);
+                           ClassTimer *T, bool per_class);
 
 // The same path on one stream (no side streams, no events); the warp-per-pair
 // kernels use warp_blocks blocks of kWarpKernelThreads threads.
