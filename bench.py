@@ -40,12 +40,9 @@ import numpy as np  # noqa: E402
 LANE_OPS_PER_CLK_PER_SM = 128
 METRIC = "BSW GCUPS on 1 GB300 (batched vs plain kernel, bit-exact); p50/p99 serve latency"
 # DRAM bytes read + written per launch of a workload's dominant kernel, from
-# one ncu capture of the current kernel (bytes, source); other kernels and
-# workloads report null.
-MEASURED_TRAFFIC = {
-    ("read250", "k_inter<128,u8>"): (49_626_624, "ncu dram__bytes_read.sum + dram__bytes_write.sum of the dominant "
-                                                 "launch, profiles/k_inter128_u8_read250.md"),
-}
+# one ncu capture of the current kernel: (workload, class) -> (bytes, source);
+# others report null.  Empty until the row-pair kernels' launch is captured alone.
+MEASURED_TRAFFIC = {}
 
 SECONDARY = ("read151", "long10k")
 
@@ -228,7 +225,8 @@ def class_of(q_len, t_len, h0, match, plan):
 
 
 def class_kernel(c, plan, scoring):
-    """Name of the kernel that runs class c under the plan."""
+    """Label of class c under the plan: "k_inter" (one pair per thread; the kernels are k_rows2 and
+    k_rows2_16) or "k_inter2" with the class's bound, or the warp or block kernel's name."""
     packable = (scoring.match + min(scoring.mismatch, 255 - scoring.match)
                 + max(min(scoring.o_del + scoring.e_del, 255), min(scoring.o_ins + scoring.e_ins, 255)) <= 256)
     if c < 8:
@@ -878,7 +876,7 @@ def run_gb300(args):
             "dtype": "u8 storage, s16x2 arithmetic (two rows per instruction)" if args.config != "long10k"
                      else "int16 storage, s16x2 arithmetic (two columns per instruction)",
             "dtype_note": "per-pair lane storage by the exact score bound h0 + match*min(n, m) (8-bit when <= 255, "
-                          "16-bit when <= 32767, else 32-bit); the 8-bit pairs without N bases compute two rows "
+                          "16-bit when <= 32767, else 32-bit); 8-bit pairs and 16-bit ones up to a bound of 2047 compute two rows "
                           "per packed s16x2 DPX instruction and the long queries' warp kernel two columns, the "
                           "other kernels in 32-bit registers; pairs whose scores leave their lane range are re-run "
                           "exactly in 32 bits",

@@ -502,7 +502,7 @@ __device__ unsigned long long x2_pair(const Batch &B, const Params &P, int p, ui
 // What bounds it: issue and the latency of a row (12 warps an SM, about 380
 // instructions a row, 93 of them the cells of a 700-column window, the rest the
 // scan, the row's decisions and the moves of the window).  20 000 pairs of up to
-// 10 kbp: 12.6 ms, against 17.7 with the ring below, which reloads and stores H
+// 10 kbp: 12.6 ms, against 17.7 with the ring above, which reloads and stores H
 // and E and finds query bases and slots anew in every row.  On the way: a
 // switch over the registers for the two band ends 14.4 ms (its branches leave
 // the instruction fetch idle); windows of 256, 512, 768 and 1024 columns 13.1
@@ -563,7 +563,7 @@ __device__ __forceinline__ void xr_scores(const XrPair &Q, const Params &P, uint
 
 // Band widths up to which the window of 512 columns is taken, and from which
 // the one of 1024 is left again (the difference keeps a band from going back
-// and forth; each change costs about ten rows).
+// and forth; each change costs the work of about ten rows).
 constexpr int kXrNarrow = 472, kXrLeave = 408;
 
 // Rows from S.i on in a window of 64 half lanes of 4 G columns.  Returns true
