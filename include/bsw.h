@@ -551,7 +551,8 @@ int bsw_sal_lookup(bsw_ctx_t *ctx, int64_t n_intervals, const int64_t *k, const 
  * index of read r's first record.  *n_out receives the number of records;
  * if it exceeds out_cap nothing is written to out and BSW_EBUDGET is
  * returned (call again with a larger out).  Device memory: about 160 bytes
- * per read besides the reads, plus 12 * (max(read_len) + 1) bytes per read
+ * per read besides the reads (about 290 for reads past 160 bases where that
+ * stays within a quarter of the budget), plus 12 * (max(read_len) + 1) bytes per read
  * whose search needs more than 24 match intervals at once.
  * bsw_smem_n also takes an N bitmap of the reads (bit p & 7 of byte p >> 3
  * marks base p as N; NULL: none): an N occurs nowhere in T, so no match

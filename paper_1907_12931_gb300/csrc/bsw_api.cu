@@ -1838,12 +1838,18 @@ int bsw_smem_n(bsw_ctx_t *ctx, int64_t n_reads, const uint8_t *reads, const uint
                      o_rlen = take(4 * (size_t)n_reads), o_cnt = take(8 * (size_t)n_reads),
                      o_first = take(8 * ((size_t)n_reads + 1)), o_ids = take(4 * (size_t)n_reads),
                      o_many = take(4 * (size_t)n_reads), o_tot = take(sizeof(SmemTotals)),
-                     o_tile = take(8 * (size_t)smem_tiles(n_reads)), o_next = take(4), o_keep = take(sizeof(uint4) * kSmemKeep * (size_t)n_reads),
+                     o_tile = take(8 * (size_t)smem_tiles(n_reads)), o_next = take(4),
                      o_rn = take(reads_n ? (size_t)((read_bytes + 1) / 2) : 0),
                      o_out = take(sizeof(bsw_smem_t) * (size_t)std::max<int64_t>(out_cap, 1));
+        // The longer keep only where the whole buffer stays within a quarter of
+        // the budget: a tight context keeps the room it had.
+        const size_t o_keep = o;
+        int32_t keep = lmax > kSmemKeepLen ? kSmemKeepLong : kSmemKeep;
+        auto after_keep = [&] { return align_up(o_keep + sizeof(uint4) * (size_t)keep * (size_t)n_reads, 256); };
+        if (after_keep() + 4 * (size_t)groups * (size_t)(starts_cap + 1) + 256 > (size_t)ctx->budget.cap / 4) keep = kSmemKeep;
         // the search starts of as many groups at a time as the budget holds
         int64_t chunk = groups;
-        size_t o_starts = o, o_nst = 0;
+        size_t o_starts = after_keep(), o_nst = 0;
         int rc;
         for (;; chunk = (chunk + 1) / 2) {
             o_nst = align_up(o_starts + 4 * (size_t)chunk * (size_t)starts_cap, 256);
@@ -1865,7 +1871,7 @@ int bsw_smem_n(bsw_ctx_t *ctx, int64_t n_reads, const uint8_t *reads, const uint
                        reads_n ? d + o_rn : nullptr};
         const SmemWork W{(int64_t *)(d + o_cnt), (uint4 *)(d + o_keep), (int64_t *)(d + o_first), (bsw_smem_t *)(d + o_out),
                          (uint32_t *)(d + o_next), (SmemTotals *)(d + o_tot), (int32_t *)(d + o_ids), (int32_t *)(d + o_many),
-                         (int64_t *)(d + o_tile), (uint32_t *)(d + o_starts), (uint32_t *)(d + o_nst), starts_cap};
+                         (int64_t *)(d + o_tile), (uint32_t *)(d + o_starts), (uint32_t *)(d + o_nst), starts_cap, keep};
         auto global_lists = [&](int64_t n_ids, BiIv **lists) -> int {      // lmax + 1 entries hold any list
             const int r2 = ctx->smemscratch.reserve(sizeof(BiIv) * (size_t)n_ids * (size_t)(lmax + 1), ctx->budget);
             *lists = (BiIv *)ctx->smemscratch.p;

@@ -29,7 +29,7 @@
 // start per lane and does its forward and backward pass.  A read with more than
 // kListCap matches in one list is finished by a launch with lists in global
 // memory (k_smem_global), where a lane does a whole read.  One pass keeps up to
-// kSmemKeep records per read in a scratch buffer; after a prefix sum of the
+// W.keep records per read in a scratch buffer; after a prefix sum of the
 // counts a gather sorts them into place, and the rare reads with more are searched
 // again, writing in place.
 #include <cuda_runtime.h>
@@ -158,8 +158,8 @@ struct ReadRef {
 };
 
 // All SMEMs of at least min_len bases of the reads t < t_end taken from the
-// counter *W.next (read ids[t]).  Store mode: count[r], and the first kSmemKeep
-// matches at scratch[r * kSmemKeep], in the order they are found
+// counter *W.next (read ids[t]).  Store mode: count[r], and the first W.keep
+// matches at scratch[r * W.keep], in the order they are found
 // (k_smem_gather sorts them); a read with more is finished by a write-mode
 // launch.  Write mode: the records at out[first[r]], in increasing start order.
 // A lane's list holds cap entries, enough for any read of the batch.
@@ -195,7 +195,7 @@ __device__ void smem_lanes(const SmemIn &R, const FmDev &F, int min_len, int64_t
     auto emit = [&](int start, int end, uint32_t k, uint32_t s) {
         if (end - start < min_len) return;
         if (WRITE) W.out[o + n] = bsw_smem_t{(int32_t)r, start, end - start, 0, (int64_t)k, (int64_t)s};
-        else if (n < kSmemKeep) W.scratch[o + n] = make_uint4((uint32_t)start, (uint32_t)(end - start), k, s);
+        else if (n < W.keep) W.scratch[o + n] = make_uint4((uint32_t)start, (uint32_t)(end - start), k, s);
         ++n;
     };
     for (;;) {
@@ -207,7 +207,7 @@ __device__ void smem_lanes(const SmemIn &R, const FmDev &F, int min_len, int64_t
                 r = ids[t];
                 L = R.read_len[r];
                 read = ReadRef(R, R.read_off[r]);
-                o = WRITE ? W.first[r] : (int64_t)r * kSmemKeep;
+                o = WRITE ? W.first[r] : (int64_t)r * W.keep;
                 n = 0;
                 x = 0;
                 state = kCall;
@@ -326,7 +326,7 @@ __device__ __forceinline__ void emit_match(const SmemWork &W, int min_len, int r
 {
     if (end - start < min_len) return;
     const unsigned long long n = atomicAdd(reinterpret_cast<unsigned long long *>(W.count + r), 1ull);
-    if (n < kSmemKeep) W.scratch[(int64_t)r * kSmemKeep + n] = make_uint4((uint32_t)start, (uint32_t)(end - start), k, s);
+    if (n < W.keep) W.scratch[(int64_t)r * W.keep + n] = make_uint4((uint32_t)start, (uint32_t)(end - start), k, s);
 }
 
 __device__ __forceinline__ void overflow_read(const SmemWork &W, int r)
@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(kFirstThreads) k_smem_sums(int64_t n_reads, Sm
     for (int u = 0; u < kFirstPer; ++u) {
         const int64_t r = (int64_t)blockIdx.x * kFirstTile + u * kFirstThreads + threadIdx.x;
         const int64_t c = r < n_reads ? W.count[r] : 0;
-        if (c > kSmemKeep) W.many[atomicAdd(&W.totals->many, 1u)] = (int32_t)r;
+        if (c > W.keep) W.many[atomicAdd(&W.totals->many, 1u)] = (int32_t)r;
         v += c;
     }
     v = block_sum(v);
@@ -590,15 +590,15 @@ __global__ void __launch_bounds__(kFirstThreads) k_smem_first(int64_t n_reads, S
     }
 }
 
-// Records of the reads with at most kSmemKeep from the scratch to out[first[r]],
+// Records of the reads with at most W.keep from the scratch to out[first[r]],
 // sorted by start (a read's SMEMs have distinct starts).
 __global__ void __launch_bounds__(256) k_smem_gather(int64_t n_reads, SmemWork W)
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n_reads; r += stride) {
         const int c = (int)W.count[r];
-        if (c > kSmemKeep) continue;
-        const uint4 *v = W.scratch + r * kSmemKeep;
+        if (c > W.keep) continue;
+        const uint4 *v = W.scratch + r * W.keep;
         for (int k = 0; k < c; ++k) {
             const uint4 u = v[k];
             int rank = 0;

@@ -237,7 +237,12 @@ struct BiIv {
     uint32_t k, s;
     int32_t e;
 };
-constexpr int kSmemThreads = 128, kListCap = 24, kSmemBlocksPerSm = 7, kSmemKeep = 8;
+constexpr int kSmemThreads = 128, kListCap = 24, kSmemBlocksPerSm = 7;
+// Records kept per read in the search pass.  A read with more is searched again by
+// one lane, 2.1 ms for a 250 bp read whatever their number, so reads past 160
+// bases keep 16 (155 949 reads of 250 bp: 3.3 ms against 4.5 a call; 200 000 of 151 bp hold at
+// most 8).
+constexpr int kSmemKeep = 8, kSmemKeepLong = 16, kSmemKeepLen = 160;
 // Search starts a group of 32 reads of at most lmax bases has room for.  Past a
 // sequencing error a search reaches about 13 bases, so twice that many fit.
 constexpr int smem_starts_cap(int lmax) { return 32 * (4 + lmax / 6); }
@@ -251,7 +256,7 @@ struct SmemTotals {
 // Buffers of one SMEM search.  Store mode: count[r] (2^40 or more, and r once in
 // ovf_list[totals->overflows++], when a list of the read exceeds kListCap or its
 // starts the group's room) and up to
-// kSmemKeep matches {start, length, k, s} at scratch[r * kSmemKeep].  Write
+// keep matches {start, length, k, s} at scratch[r * keep].  Write
 // mode: records at out[first[r]].  next: the launch's read counter (zeroed by the launchers).
 struct SmemWork {
     int64_t *count;
@@ -261,11 +266,12 @@ struct SmemWork {
     uint32_t *next;
     SmemTotals *totals;
     int32_t *ovf_list;
-    int32_t *many;           // reads with more than kSmemKeep records (totals->many)
+    int32_t *many;           // reads with more than keep records (totals->many)
     int64_t *tile_sum;       // [smem_tiles(n_reads)]
     uint32_t *starts;        // [groups of 32 reads][starts_cap] search starts: start | lane << 16
     uint32_t *n_starts;      // [groups]: the starts noted
     int32_t starts_cap;
+    int32_t keep;            // kSmemKeep or kSmemKeepLong
 };
 // W.starts and W.n_starts hold `chunk` groups; the reads are searched in as
 // many rounds as that takes.
@@ -275,11 +281,11 @@ cudaError_t launch_smem_store(const SmemIn &R, const FmDev &F, int min_len, cons
 // entries per lane, n_ids lanes at most).
 cudaError_t launch_smem_global(bool write, const SmemIn &R, const FmDev &F, int min_len, const SmemWork &W,
                                const int32_t *ids, int64_t n_ids, BiIv *lists, int cap, cudaStream_t st, int sms);
-// first[] from the counts, the reads with more than kSmemKeep records, and the
+// first[] from the counts, the reads with more than keep records, and the
 // number of records (totals).
 int64_t smem_tiles(int64_t n_reads);
 cudaError_t launch_smem_first(int64_t n_reads, const SmemWork &W, cudaStream_t st);
-// Records of reads with count <= kSmemKeep from the scratch to out[first[r]].
+// Records of reads with count <= keep from the scratch to out[first[r]].
 cudaError_t launch_smem_gather(int64_t n_reads, const SmemWork &W, cudaStream_t st, int sms);
 
 // Suffix array lookup: out[off[t] + i] = sa[k[t] + i] for i < cnt[t].

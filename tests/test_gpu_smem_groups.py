@@ -83,3 +83,24 @@ def test_rounds_under_a_tight_budget(bsw):
         if done == 12:
             break
     assert done >= 3
+
+
+@pytest.mark.parametrize("lmax,budget", [(160, 1 << 30), (161, 1 << 30), (300, 1 << 30), (300, 3 << 20)])
+def test_reads_with_many_records(bsw, lmax, budget):
+    """Counts on both sides of the records a read keeps (8, or 16 past 160
+    bases and with room in the budget): the others are searched again."""
+    rng = np.random.default_rng(lmax)
+    ref = rng.integers(0, 4, 3000).astype(np.uint8)
+    reads = []
+    for k in range(200):
+        p = int(rng.integers(0, len(ref) - lmax))
+        x = ref[p:p + lmax].copy()
+        at = rng.choice(lmax, int(rng.integers(0, 24)), replace=False)
+        x[at] = (x[at] + 1) % 4
+        reads.append(np.ascontiguousarray(3 - x[::-1]) if k & 1 else x)
+    want = expected(ref, reads, 8)
+    counts = [len(r) for r in want]
+    assert min(counts) <= 8 < max(counts) and max(counts) > 16
+    with bsw.Context(W.Params(), budget) as ctx:
+        ctx.fm_build(ref)
+        assert search(bsw, ctx, reads, 8) == want
