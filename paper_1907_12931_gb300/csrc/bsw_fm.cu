@@ -21,7 +21,8 @@
 // those matches backward one base at a time, longest first.  A match that can
 // no longer be extended while no longer one survives at that base is an SMEM.
 // The next x is the end of the longest match from x; every SMEM holds exactly
-// one of the visited x.
+// one of the visited x.  No search starts at an N or at a base that T does not
+// hold: no match contains either.
 //
 // The starts x depend on the forward searches alone, so the search is cut in
 // two kernels whose lanes do the same work at the same time: k_smem_scan takes
@@ -142,6 +143,12 @@ __device__ __forceinline__ uint32_t first_row(const FmDev &F, int c)
     return c < 2 ? (c == 0 ? F.C[0] : F.C[1]) : c == 2 ? F.C[2] : c == 3 ? F.C[3] : F.C[4];
 }
 
+// Whether a search can start at base c (4: N): the text holds it.
+__device__ __forceinline__ bool in_text(const FmDev &F, int c)
+{
+    return c < 4 && first_row(F, c + 1) != first_row(F, c);
+}
+
 // A read of the batch: its packed bases (a read starts on a byte) and its base
 // offset, which addresses the N bitmap.
 struct ReadRef {
@@ -218,7 +225,7 @@ __device__ void smem_lanes(const SmemIn &R, const FmDev &F, int min_len, int64_t
                     continue;
                 }
                 const int c0 = base_at(x);
-                if (c0 > 3) {                                           // no match starts at an N
+                if (!in_text(F, c0)) {
                     ++x;
                     continue;
                 }
@@ -361,9 +368,9 @@ __global__ void __launch_bounds__(kSmemThreads) k_smem_scan(SmemIn R, FmDev F, i
         const uint32_t b = 3u - (uint32_t)(c & 3);
         const Ext u = extend(F, vl, vs, b);
         const uint32_t s2 = c < 4 ? u.size : 0u;
-        const bool ends = i < L && x >= 0 && s2 == 0 && vs > 0;
+        const bool ends = i < L && x >= 0 && s2 == 0;
         if (ends && x == 0) emit_match(W, min_len, r, 0, i, vk, vs);
-        const bool starts_here = i < L && (x < 0 || ends) && c < 4;     // no match starts at an N
+        const bool starts_here = i < L && (x < 0 || ends) && in_text(F, c);
         if (starts_here) {
             vk = first_row(F, c);
             vl = first_row(F, 3 - c);
@@ -434,7 +441,7 @@ __global__ void __launch_bounds__(kSmemThreads) k_smem_store(SmemIn R, FmDev F, 
                 x = (int)(st & 0xffffu);
                 read = ReadRef(R, R.read_off[r]);
                 L = R.read_len[r];
-                c = read.base(R, x);                                     // a base: no search starts at an N
+                c = read.base(R, x);                                     // a base of the text
                 cpos = x;
                 vk = first_row(F, c);
                 vl = first_row(F, 3 - c);

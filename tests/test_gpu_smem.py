@@ -128,3 +128,24 @@ def test_reads_with_n(bsw):
         for r, w in enumerate(want):
             g = got[first[r]:first[r + 1]]
             assert [tuple(int(v) for v in x) for x in g[["qbeg", "len", "k", "s"]]] == [tuple(x) for x in w], r
+
+
+@pytest.mark.parametrize("codes", [(0,), (1, 2), (0, 3)])
+def test_bases_the_text_does_not_hold(bsw, codes):
+    """A text of one base and its complement: a read base that occurs in
+    neither strand is in no match, at a read's start, inside it and in runs.
+    Reads with few records, reads whose lists overflow (a repeat of one base)
+    and reads with more records than the first pass keeps."""
+    rng = np.random.default_rng(400 + codes[0])
+    ref = rng.choice(codes, 400).astype(np.uint8)
+    other = [c for c in range(4) if c not in codes and 3 - c not in codes]
+    reads = [np.array([other[0]] + [codes[0]] * 7, np.uint8), np.array(other * 3, np.uint8)]
+    for k in range(60):
+        L = int(rng.integers(1, 80))
+        p = int(rng.integers(0, ref.shape[0] - L))
+        x = ref[p:p + L].copy()
+        x[rng.random(L) < (0.02, 0.1, 0.4)[k % 3]] = other[k % len(other)]
+        reads.append(np.ascontiguousarray(3 - x[::-1]) if k & 1 else x)
+    reads.append(np.where(np.arange(150) % 4 == 0, other[0], ref[:150]).astype(np.uint8))   # 38 of them
+    for min_len in (1, 5):
+        check(bsw, ref, reads, min_len)
