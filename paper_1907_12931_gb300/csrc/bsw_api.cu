@@ -1908,13 +1908,19 @@ int bsw_smem_n(bsw_ctx_t *ctx, int64_t n_reads, const uint8_t *reads, const uint
             if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_rc(e);
             return total == 0 ? BSW_OK : BSW_EBUDGET;
         }
-        if ((e = launch_smem_gather(n_reads, W, st, ctx->sms)) != cudaSuccess) return cuda_rc(e);
+        // the copy into the caller's first[] is on its way, which a pinned array
+        // shows: no return before it is done
+        auto leave = [&](int code) {
+            const cudaError_t le = cudaStreamSynchronize(st);
+            return le != cudaSuccess ? cuda_rc(le) : code;
+        };
+        if ((e = launch_smem_gather(n_reads, W, st, ctx->sms)) != cudaSuccess) return leave(cuda_rc(e));
         if (n_many > 0) {
             BiIv *lists = nullptr;
-            if ((rc = global_lists(n_many, &lists)) != BSW_OK) return rc;
+            if ((rc = global_lists(n_many, &lists)) != BSW_OK) return leave(rc);
             if ((e = launch_smem_global(true, R, ctx->fm_t, min_len, W, W.many, n_many, lists, lmax + 1, st, ctx->sms)) !=
                 cudaSuccess)
-                return cuda_rc(e);
+                return leave(cuda_rc(e));
         }
         if ((e = cudaMemcpyAsync(out, W.out, sizeof(bsw_smem_t) * (size_t)total, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
             (e = cudaStreamSynchronize(st)) != cudaSuccess)

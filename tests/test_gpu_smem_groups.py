@@ -104,3 +104,46 @@ def test_reads_with_many_records(bsw, lmax, budget):
     with bsw.Context(W.Params(), budget) as ctx:
         ctx.fm_build(ref)
         assert search(bsw, ctx, reads, 8) == want
+
+
+def test_refused_lists_leave_nothing_in_flight(bsw):
+    """A call that cannot hold the lists of the reads with many records returns
+    with first[] complete, also when it is pinned and the device writes it."""
+    import torch
+    rng = np.random.default_rng(9)
+    ref = rng.integers(0, 4, 3000).astype(np.uint8)
+    n = 2_000_000                                                  # 16 MB of first[]
+    reads = []
+    for _ in range(300):
+        p = int(rng.integers(0, 2400))
+        x = ref[p:p + 600].copy()
+        x[::12] = (x[::12] + 1) % 4                                # some 50 records
+        reads.append(x)
+    reads.append(rng.integers(0, 4, 32768).astype(np.uint8))       # room for 32769 matches a list
+    ln = np.zeros(n, np.int32)
+    ln[:len(reads)] = [len(x) for x in reads]
+    off, total = W.layout(ln, 4)
+    codes = np.zeros(total, np.uint8)
+    for o, x in zip(off, reads):
+        codes[o:o + len(x)] = x
+    packed = bsw.bsw_pack_2bit(codes)
+    out, found = np.zeros(100_000, bsw.SMEM_DTYPE), np.zeros(1, np.int64)
+    first = torch.full((n + 1,), -1, dtype=torch.int64).pin_memory()
+    f = first.numpy()
+
+    def call(ctx):
+        return bsw.lib().bsw_smem(ctx.handle, n, packed.ctypes.data, off.ctypes.data, ln.ctypes.data, 10,
+                                  out.ctypes.data, out.shape[0], found.ctypes.data, f.ctypes.data)
+
+    with bsw.Context(W.Params(), 4 << 30) as ctx:
+        ctx.fm_build(ref)
+        assert call(ctx) == bsw.BSW_OK
+    want = f.copy()
+    with bsw.Context(W.Params(), 400 << 20) as ctx:
+        ctx.fm_build(ref)
+        for _ in range(5):
+            first.fill_(-1)
+            assert call(ctx) == bsw.BSW_EBUDGET                    # 300 lists of 32769 entries: 118 MB
+            last = int(f[n])
+            assert last == found[0] == want[n]
+            np.testing.assert_array_equal(f, want)
