@@ -222,10 +222,12 @@ int bsw_stream_poll(bsw_ctx_t *ctx, uint64_t ticket, int32_t timeout_us);
  * fail as if the runtime had refused it, so the caller sees the documented
  * code and the context must stay usable afterwards.  Sites:
  *   alloc   a device (cudaMalloc) or pinned host (cudaMallocHost) allocation
- *           of a context's buffers: the call returns BSW_ENOMEM
+ *           of a context's buffers: the call returns BSW_ENOMEM, unless it can
+ *           do with less (see bsw_smem's memory)
  *   h2d     a host-to-device copy of a host batch (bsw_extend_batch with host
  *           pointers, the serving loop's staging): BSW_ECUDA
- *   launch  the launch of a batch's kernels: BSW_ECUDA
+ *   launch  the launch of a batch's kernels, or of a round of an SMEM search:
+ *           BSW_ECUDA
  *   thread  the start of a context's serving thread: bsw_stream_submit
  *           returns BSW_ENOMEM and registers nothing
  *   host    a host container allocation in the serving path (ticket table,
@@ -550,10 +552,17 @@ int bsw_sal_lookup(bsw_ctx_t *ctx, int64_t n_intervals, const int64_t *k, const 
  * suffix array of T.  first[r] (n_reads + 1 entries, nullable) receives the
  * index of read r's first record.  *n_out receives the number of records;
  * if it exceeds out_cap nothing is written to out and BSW_EBUDGET is
- * returned (call again with a larger out).  Device memory: about 160 bytes
- * per read besides the reads (about 290 for reads past 160 bases where that
- * stays within a quarter of the budget), plus 12 * (max(read_len) + 1) bytes per read
- * whose search needs more than 24 match intervals at once.
+ * returned (call again with a larger out).  Device memory besides the reads
+ * and out_cap records:
+ *   - about 165 bytes per read (295 in a batch with reads past 160 bases where
+ *     that stays within a quarter of the budget);
+ *   - the starts of the searches, 4 * (4 + read_len / 6) bytes per read, of all
+ *     reads at once where these stay within a quarter of the budget, else of as
+ *     many as fit, in rounds (of the longest read at least).  The context keeps
+ *     this buffer and gives it up where another call's memory would be refused;
+ *   - 12 * (max(read_len) + 1) bytes per read whose search needs more than 24
+ *     match intervals at once or that has more than 8 records (16 in the batches
+ *     of 295 bytes).
  * bsw_smem_n also takes an N bitmap of the reads (bit p & 7 of byte p >> 3
  * marks base p as N; NULL: none): an N occurs nowhere in T, so no match
  * contains one.

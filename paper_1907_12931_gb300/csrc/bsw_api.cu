@@ -45,9 +45,16 @@ constexpr int kGraphCache = 8;
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+struct DevBuf;
+
 struct Budget {
     int64_t cap = 0;
     std::atomic<int64_t> used{0};
+    // A buffer that no call needs once it has returned: it is given up where
+    // another reservation would be refused.  spare_mu is held while it is in use.
+    DevBuf *spare = nullptr;
+    std::mutex spare_mu;
+    bool drop_spare();
 };
 
 // ---------------------------------------------------------- fault injection
@@ -155,6 +162,11 @@ struct DevBuf {
 
     int reserve(size_t bytes, Budget &B, bool *moved = nullptr)
     {
+        const int rc = grow(bytes, B, moved);
+        return rc != BSW_OK && B.drop_spare() ? grow(bytes, B, moved) : rc;
+    }
+    int grow(size_t bytes, Budget &B, bool *moved = nullptr)
+    {
         if (bytes <= cap) return BSW_OK;
         size_t want = align_up(std::max(bytes, cap + cap / 4), 1 << 20);
         if (B.used.load() - (int64_t)cap + (int64_t)want > B.cap) want = align_up(bytes, 256);
@@ -181,6 +193,14 @@ struct DevBuf {
         cap = 0;
     }
 };
+
+bool Budget::drop_spare()
+{
+    std::lock_guard<std::mutex> lk(spare_mu);
+    if (!spare || !spare->p) return false;
+    spare->release(*this);
+    return true;
+}
 
 // Byte offsets of the work buffers inside one allocation.
 struct WorkLayout {
@@ -444,9 +464,10 @@ struct bsw_ctx {
     DevBuf sabuf, salio;
     int64_t sa_n = -1;
 
-    // SMEM search: the FM-index of T = ref + revcomp(ref); staging, and the
-    // global lists of reads whose lists overflow shared memory
-    DevBuf fmbuf, smemio, smemscratch;
+    // SMEM search: the FM-index of T = ref + revcomp(ref); staging, the search
+    // starts (budget.spare), and the global lists of reads whose lists overflow
+    // shared memory
+    DevBuf fmbuf, smemio, smemstarts, smemscratch;
     FmDev fm_t{};
     bool fm_ready = false;
 
@@ -1087,6 +1108,7 @@ int bsw_init(const bsw_scoring_t *sc, int32_t w, int32_t zdrop, int32_t end_bonu
     c->P = Params{sc->match, sc->mismatch, sc->o_del, sc->e_del, sc->o_ins, sc->e_ins, w, zdrop, end_bonus, 0u, kLongMax,
                   1u << 8, 1u << 16, 1u << 24, kShortMax};
     c->budget.cap = mem_budget_bytes;
+    c->budget.spare = &c->smemstarts;
     int rc = BSW_OK;
     if (cudaGetDevice(&c->device) != cudaSuccess ||
         cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) {
@@ -1819,59 +1841,69 @@ int bsw_smem_n(bsw_ctx_t *ctx, int64_t n_reads, const uint8_t *reads, const uint
         if (n_reads == 0) return BSW_OK;
         // branch-free, so that the compiler vectorises it (200 k reads: 175 us with
         // an early return per read)
-        int64_t bases_end = 0;
+        int64_t bases_end = 0, bases = 0;
         int32_t lmax = 0, bad = 0;
         for (int64_t r = 0; r < n_reads; ++r) {
             const int64_t off = read_off[r];
             const int32_t len = read_len[r];
             bad |= (int32_t)(off < 0) | (int32_t)(off & 3) | (int32_t)(len < 0) | (int32_t)(len > kLongMax);
             bases_end = std::max(bases_end, (int64_t)((uint64_t)off + (uint64_t)(int64_t)len));
+            bases += len;
             lmax = std::max(lmax, len);
         }
         if (bad) return BSW_EINVAL;
         const int64_t read_bytes = (bases_end + 3) / 4;
         size_t o = 0;
         auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes, 256); return r; };
-        const int64_t groups = (n_reads + 31) / 32;
-        const int starts_cap = smem_starts_cap(lmax);
         const size_t o_reads = take((size_t)read_bytes), o_roff = take(8 * (size_t)n_reads),
                      o_rlen = take(4 * (size_t)n_reads), o_cnt = take(8 * (size_t)n_reads),
                      o_first = take(8 * ((size_t)n_reads + 1)), o_ids = take(4 * (size_t)n_reads),
                      o_many = take(4 * (size_t)n_reads), o_tot = take(sizeof(SmemTotals)),
-                     o_tile = take(8 * (size_t)smem_tiles(n_reads)), o_next = take(4),
+                     o_tile = take(8 * (size_t)smem_tiles(n_reads)), o_ctr = take(sizeof(SmemCounters)),
+                     o_group = take(sizeof(SmemGroup) * (size_t)((n_reads + 31) / 32)),
                      o_rn = take(reads_n ? (size_t)((read_bytes + 1) / 2) : 0),
                      o_out = take(sizeof(bsw_smem_t) * (size_t)std::max<int64_t>(out_cap, 1));
         // The longer keep only where the whole buffer stays within a quarter of
         // the budget: a tight context keeps the room it had.
-        const size_t o_keep = o;
         int32_t keep = lmax > kSmemKeepLen ? kSmemKeepLong : kSmemKeep;
-        auto after_keep = [&] { return align_up(o_keep + sizeof(uint4) * (size_t)keep * (size_t)n_reads, 256); };
-        if (after_keep() + 4 * (size_t)groups * (size_t)(starts_cap + 1) + 256 > (size_t)ctx->budget.cap / 4) keep = kSmemKeep;
-        // the search starts of as many groups at a time as the budget holds
-        int64_t chunk = groups;
-        size_t o_starts = after_keep(), o_nst = 0;
-        int rc;
-        for (;; chunk = (chunk + 1) / 2) {
-            o_nst = align_up(o_starts + 4 * (size_t)chunk * (size_t)starts_cap, 256);
-            rc = ctx->smemio.reserve(o_nst + 4 * (size_t)chunk, ctx->budget);
-            if (rc != BSW_EBUDGET || chunk == 1) break;
-        }
+        auto total_bytes = [&] { return o + sizeof(uint4) * (size_t)keep * (size_t)n_reads; };
+        if (total_bytes() > (size_t)ctx->budget.cap / 4) keep = kSmemKeep;
+        int rc = ctx->smemio.reserve(total_bytes(), ctx->budget);
         if (rc != BSW_OK) return rc;
+
+        // Room for the search starts of all reads, if it is within a quarter of
+        // the budget, else for those of as many as it holds: the reads are then
+        // searched in rounds.  The least is the longest read's; if even that is
+        // refused, an earlier call's lists go.
+        const int64_t room_all = 4 * n_reads + bases / 6, room_one = smem_room(lmax);
+        int64_t pool = std::min(room_all, std::max(room_one, ctx->budget.cap / 16));
+        std::unique_lock<std::mutex> starts_in_use(ctx->budget.spare_mu);
+        while ((rc = ctx->smemstarts.grow(sizeof(uint32_t) * (size_t)pool, ctx->budget)) != BSW_OK) {
+            if (pool > room_one) pool = std::max(room_one, pool / 2);
+            else if (ctx->smemscratch.p) ctx->smemscratch.release(ctx->budget);
+            else return rc;
+        }
         uint8_t *d = ctx->smemio.p;
         cudaStream_t st = ctx->sync.S.main;
         cudaError_t e;
+        // every return from here on waits for the stream, which reads the caller's
+        // arrays and writes first[]
+        auto leave = [&](int code) {
+            const cudaError_t le = cudaStreamSynchronize(st);
+            return le != cudaSuccess ? cuda_rc(le) : code;
+        };
         if ((e = cudaMemcpyAsync(d + o_reads, reads, (size_t)read_bytes, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
             (e = cudaMemcpyAsync(d + o_roff, read_off, 8 * (size_t)n_reads, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
             (e = cudaMemcpyAsync(d + o_rlen, read_len, 4 * (size_t)n_reads, cudaMemcpyHostToDevice, st)) != cudaSuccess)
-            return cuda_rc(e);
+            return leave(cuda_rc(e));
         if (reads_n && read_bytes &&
             (e = cudaMemcpyAsync(d + o_rn, reads_n, (size_t)((read_bytes + 1) / 2), cudaMemcpyHostToDevice, st)) != cudaSuccess)
-            return cuda_rc(e);
+            return leave(cuda_rc(e));
         const SmemIn R{d + o_reads, (const int64_t *)(d + o_roff), (const int32_t *)(d + o_rlen), n_reads, lmax,
                        reads_n ? d + o_rn : nullptr};
-        const SmemWork W{(int64_t *)(d + o_cnt), (uint4 *)(d + o_keep), (int64_t *)(d + o_first), (bsw_smem_t *)(d + o_out),
-                         (uint32_t *)(d + o_next), (SmemTotals *)(d + o_tot), (int32_t *)(d + o_ids), (int32_t *)(d + o_many),
-                         (int64_t *)(d + o_tile), (uint32_t *)(d + o_starts), (uint32_t *)(d + o_nst), starts_cap, keep};
+        const SmemWork W{(int64_t *)(d + o_cnt), (uint4 *)(d + o), (int64_t *)(d + o_first), (bsw_smem_t *)(d + o_out),
+                         (SmemCounters *)(d + o_ctr), (SmemTotals *)(d + o_tot), (int32_t *)(d + o_ids), (int32_t *)(d + o_many),
+                         (int64_t *)(d + o_tile), (uint32_t *)ctx->smemstarts.p, (SmemGroup *)(d + o_group), keep};
         auto global_lists = [&](int64_t n_ids, BiIv **lists) -> int {      // lmax + 1 entries hold any list
             const int r2 = ctx->smemscratch.reserve(sizeof(BiIv) * (size_t)n_ids * (size_t)(lmax + 1), ctx->budget);
             *lists = (BiIv *)ctx->smemscratch.p;
@@ -1889,31 +1921,34 @@ int bsw_smem_n(bsw_ctx_t *ctx, int64_t n_reads, const uint8_t *reads, const uint
                 return cuda_rc(pe);
             return BSW_OK;
         };
-        if ((e = launch_smem_store(R, ctx->fm_t, min_len, W, chunk, st, ctx->sms)) != cudaSuccess) return cuda_rc(e);
-        if ((rc = positions()) != BSW_OK) return rc;
+        if ((e = launch_smem_clear(n_reads, W, st)) != cudaSuccess) return leave(cuda_rc(e));
+        for (int64_t r0 = 0, r1 = 0; r0 < n_reads; r0 = r1) {
+            if (room_all <= pool) {
+                r1 = n_reads;
+            } else {
+                int64_t room = smem_room(read_len[r1++]);
+                while (r1 < n_reads && room + smem_room(read_len[r1]) <= pool) room += smem_room(read_len[r1++]);
+            }
+            if (fault_hit(BSW_FAULT_LAUNCH)) return leave(BSW_ECUDA);
+            if ((e = launch_smem_store(R, ctx->fm_t, min_len, W, r0, r1 - r0, st, ctx->sms)) != cudaSuccess)
+                return leave(cuda_rc(e));
+        }
+        if ((rc = positions()) != BSW_OK) return leave(rc);
+        starts_in_use.unlock();
         const int64_t n_ovf = ctx->h_smem->overflows;
         if (n_ovf > 0) {
             BiIv *lists = nullptr;
             if ((rc = global_lists(n_ovf, &lists)) != BSW_OK) return rc;
             if ((e = launch_smem_global(false, R, ctx->fm_t, min_len, W, W.ovf_list, n_ovf, lists, lmax + 1, st, ctx->sms)) !=
                 cudaSuccess)
-                return cuda_rc(e);
-            if ((rc = positions()) != BSW_OK) return rc;
+                return leave(cuda_rc(e));
+            if ((rc = positions()) != BSW_OK) return leave(rc);
         }
         const int64_t total = ctx->h_smem->records, n_many = ctx->h_smem->many;
         *n_out = total;
         if (first && (e = cudaMemcpyAsync(first, W.first, 8 * ((size_t)n_reads + 1), cudaMemcpyDeviceToHost, st)) != cudaSuccess)
-            return cuda_rc(e);
-        if (total == 0 || total > out_cap) {
-            if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_rc(e);
-            return total == 0 ? BSW_OK : BSW_EBUDGET;
-        }
-        // the copy into the caller's first[] is on its way, which a pinned array
-        // shows: no return before it is done
-        auto leave = [&](int code) {
-            const cudaError_t le = cudaStreamSynchronize(st);
-            return le != cudaSuccess ? cuda_rc(le) : code;
-        };
+            return leave(cuda_rc(e));
+        if (total == 0 || total > out_cap) return leave(total == 0 ? BSW_OK : BSW_EBUDGET);
         if ((e = launch_smem_gather(n_reads, W, st, ctx->sms)) != cudaSuccess) return leave(cuda_rc(e));
         if (n_many > 0) {
             BiIv *lists = nullptr;
@@ -1922,10 +1957,9 @@ int bsw_smem_n(bsw_ctx_t *ctx, int64_t n_reads, const uint8_t *reads, const uint
                 cudaSuccess)
                 return leave(cuda_rc(e));
         }
-        if ((e = cudaMemcpyAsync(out, W.out, sizeof(bsw_smem_t) * (size_t)total, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-            (e = cudaStreamSynchronize(st)) != cudaSuccess)
-            return cuda_rc(e);
-        return BSW_OK;
+        if ((e = cudaMemcpyAsync(out, W.out, sizeof(bsw_smem_t) * (size_t)total, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
+            return leave(cuda_rc(e));
+        return leave(BSW_OK);
     });
 }
 
@@ -1950,6 +1984,7 @@ void bsw_destroy(bsw_ctx_t *ctx)
     ctx->salio.release(ctx->budget);
     ctx->fmbuf.release(ctx->budget);
     ctx->smemio.release(ctx->budget);
+    ctx->smemstarts.release(ctx->budget);
     ctx->smemscratch.release(ctx->budget);
     if (ctx->timer_ready)
         for (int k = 0; k <= kNumClass; ++k) {

@@ -7,13 +7,13 @@
 // pair of their suffix-array intervals (the bi-interval [k, l, s] of
 // Algorithms 2-3) can be extended by one base on either side.
 //
-// O (Algorithm 1) is kept in buckets of eta = 32 BWT positions: entry t holds
-// the counts of each base in BWT[0, 32t) and the 32 BWT bases of the bucket,
-// 2-bit packed in one 64-bit word: 32 bytes, one DRAM sector per lookup (the
-// paper's CPU layout uses 64-byte entries with a byte per base for AVX2
-// compares; a 2-bit word and population counts serve the GPU).  One lookup
-// gives the occurrences of all four bases; the $ row is stored as base 0 and
-// subtracted.
+// O (Algorithm 1) is kept in buckets of eta = 32 BWT positions: entry t holds,
+// for each base, its first row plus its count in BWT[0, 32t), and the low and
+// the high bits of the bucket's 32 BWT bases as one 32-bit word each: 32 bytes,
+// one DRAM sector per lookup (the paper's CPU layout uses 64-byte entries with a
+// byte per base for AVX2 compares; bit planes and population counts serve the
+// GPU).  One lookup gives a base's row and the occurrences of the larger ones;
+// the $ row is stored as base 0 and subtracted.
 //
 // SMEMs of a read X (Li 2012; Algorithm 4): from a position x, extend X[x]
 // forward base by base, keeping the match each time its number of occurrences
@@ -27,7 +27,8 @@
 // The starts x depend on the forward searches alone, so the search is cut in
 // two kernels whose lanes do the same work at the same time: k_smem_scan takes
 // a read per lane, one base per step, and notes the starts; k_smem_store takes a
-// start per lane and does its forward and backward pass.  A read with more than
+// start per lane and does its forward and backward pass.  Where the budget does
+// not hold the starts of all reads at once they run in rounds.  A read with more than
 // kListCap matches in one list is finished by a launch with lists in global
 // memory (k_smem_global), where a lane does a whole read.  One pass keeps up to
 // W.keep records per read in a scratch buffer; after a prefix sum of the
@@ -165,11 +166,11 @@ struct ReadRef {
 };
 
 // All SMEMs of at least min_len bases of the reads t < t_end taken from the
-// counter *W.next (read ids[t]).  Store mode: count[r], and the first W.keep
+// counter W.ctr->next (read ids[t]).  Store mode: count[r], and the first W.keep
 // matches at scratch[r * W.keep], in the order they are found
 // (k_smem_gather sorts them); a read with more is finished by a write-mode
 // launch.  Write mode: the records at out[first[r]], in increasing start order.
-// A lane's list holds cap entries, enough for any read of the batch.
+// A lane's list holds any read of the batch.
 //
 // The lane is a small state machine so that every pass of the main loop makes
 // exactly one extension on every lane that has work (the memory lookups of
@@ -189,7 +190,7 @@ struct ReadRef {
 // needs no more than the rows, as no forward extension follows.
 template <bool WRITE>
 __device__ void smem_lanes(const SmemIn &R, const FmDev &F, int min_len, int64_t t_end, const int32_t *ids,
-                           BiIv *list, int cap, const SmemWork &W)
+                           BiIv *list, const SmemWork &W)
 {
     enum { kRead, kCall, kBack, kEnd, kFwd, kBwd };
     int state = kRead;
@@ -209,7 +210,7 @@ __device__ void smem_lanes(const SmemIn &R, const FmDev &F, int min_len, int64_t
         // settle: run the bookkeeping up to the next extension
         while (state < kFwd) {
             if (state == kRead) {
-                const int64_t t = atomicAdd(W.next, 1u);
+                const int64_t t = atomicAdd(&W.ctr->next, 1u);
                 if (t >= t_end) return;
                 r = ids[t];
                 L = R.read_len[r];
@@ -342,23 +343,27 @@ __device__ __forceinline__ void overflow_read(const SmemWork &W, int r)
         W.ovf_list[atomicAdd(&W.totals->overflows, 1u)] = r;
 }
 
-// The starts of the searches of groups [g0, g0 + ng): a warp takes 32 reads, a lane one of
-// them, a base per step.  The longest match from the read's start is an SMEM;
-// the other starts go to the group's part of W.starts (start | lane << 16).
-__global__ void __launch_bounds__(kSmemThreads) k_smem_scan(SmemIn R, FmDev F, int min_len, SmemWork W, int64_t g0, int64_t ng)
+// The starts of the searches of reads [r0, r0 + nr): a warp takes 32 of them, a
+// lane one, a base per step.  The longest match from the read's start is an SMEM;
+// the other starts go to the group's part of W.starts (start | lane << 16), which
+// has the reads' own room: one long read among short ones takes no other group's.
+__global__ void __launch_bounds__(kSmemThreads) k_smem_scan(SmemIn R, FmDev F, int min_len, SmemWork W, int64_t r0, int64_t nr)
 {
     constexpr unsigned kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1u;
     const int64_t g = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (g >= ng) return;
-    const int64_t r64 = (g0 + g) * 32 + lane;
-    const int r = (int)r64;
-    const bool mine = r64 < R.n_reads;
+    if (g * 32 >= nr) return;
+    const int r = (int)(r0 + g * 32 + lane);
+    const bool mine = g * 32 + lane < nr;
     const int L = mine ? R.read_len[r] : 0;
     ReadRef read;
     if (mine) read = ReadRef(R, R.read_off[r]);
-    uint32_t *starts = W.starts + g * W.starts_cap;
+    const unsigned room = __reduce_add_sync(kAll, mine ? (unsigned)smem_room(L) : 0u);
+    unsigned long long part = 0;
+    if (lane == 0) part = atomicAdd(&W.ctr->used, (unsigned long long)room);
+    part = __shfl_sync(kAll, part, 0);
+    uint32_t *starts = W.starts + part;
     uint32_t quad = 0;
     int i = 0, x = -1, n = 0;                // the next base; the search's start (-1: none); starts noted
     uint32_t vk = 0, vl = 0, vs = 0;         // the match X[x..i), its rows and those of its reverse complement
@@ -383,7 +388,7 @@ __global__ void __launch_bounds__(kSmemThreads) k_smem_scan(SmemIn R, FmDev F, i
         const unsigned st = __ballot_sync(kAll, starts_here && i > 0);
         if (starts_here && i > 0) {
             const int at = n + __popc(st & below);
-            if (at < W.starts_cap) starts[at] = (uint32_t)i | ((uint32_t)lane << 16);
+            if (at < (int)room) starts[at] = (uint32_t)i | ((uint32_t)lane << 16);
             else overflow_read(W, r);
         }
         n += __popc(st);
@@ -394,8 +399,9 @@ __global__ void __launch_bounds__(kSmemThreads) k_smem_scan(SmemIn R, FmDev F, i
             vl = vs = 0;                                                  // done: look up row 0
         }
     }
-    if (lane == 0) W.n_starts[g] = (uint32_t)min(n, W.starts_cap);
+    if (lane == 0) W.group[g] = SmemGroup{(int64_t)part, min(n, (int)room), 0};
 }
+
 // The searches from the noted starts: a warp works through the starts of
 // groups of 32 reads, its lanes taking the next one as they finish.  A lane's
 // matches lie in shared memory, 10 bytes each: rows and end (the rows of
@@ -407,14 +413,15 @@ __global__ void __launch_bounds__(kSmemThreads) k_smem_scan(SmemIn R, FmDev F, i
 // 25 and 18 of 32 lanes active; one kernel with a lane per read, lists of 16-byte
 // entries and two loads per bucket took 1.84 ms at 15 lanes.  24 matches a lane
 // and 7 blocks an SM run as fast as 28 and 6, 1% faster than 20 and 8.
-__global__ void __launch_bounds__(kSmemThreads) k_smem_store(SmemIn R, FmDev F, int min_len, SmemWork W, int64_t g0, int64_t ng)
+__global__ void __launch_bounds__(kSmemThreads) k_smem_store(SmemIn R, FmDev F, int min_len, SmemWork W, int64_t r0, int64_t ng)
 {
     constexpr unsigned kAll = 0xffffffffu;
     __shared__ uint2 ks[kListCap * kSmemThreads];
     __shared__ uint16_t ends[kListCap * kSmemThreads];
     const int lane = threadIdx.x & 31, me = threadIdx.x;
     const unsigned below = (1u << lane) - 1u;
-    int64_t g = 0;                           // the warp's group of reads, its starts and the next of them
+    int64_t rg = 0;                          // the first read of the warp's group, its starts and the next of them
+    const uint32_t *starts = W.starts;
     int nq = 0, head = 0;
     bool left = true;                        // groups are left
     int r = -1, L = 0, x = 0, i = 0, j = 0;  // the lane's read (-1: none), the search's start; the next base either way
@@ -426,18 +433,23 @@ __global__ void __launch_bounds__(kSmemThreads) k_smem_store(SmemIn R, FmDev F, 
     for (;;) {
         if (head == nq && left) {
             uint32_t t = 0;
-            if (lane == 0) t = atomicAdd(W.next, 1u);
-            g = (int64_t)__shfl_sync(kAll, t, 0);
+            if (lane == 0) t = atomicAdd(&W.ctr->next, 1u);
+            const int64_t g = (int64_t)__shfl_sync(kAll, t, 0);
             left = g < ng;
-            nq = left ? (int)W.n_starts[g] : 0;
-            head = 0;
+            nq = head = 0;
+            if (left) {
+                const SmemGroup G = W.group[g];
+                rg = r0 + g * 32;
+                starts = W.starts + G.at;
+                nq = G.n;
+            }
         }
         const unsigned want = __ballot_sync(kAll, r < 0);
         if (want && head < nq) {
             const int t = head + __popc(want & below);
             if (r < 0 && t < nq) {
-                const uint32_t st = W.starts[g * W.starts_cap + t];
-                r = (int)((g0 + g) * 32 + (st >> 16));
+                const uint32_t st = starts[t];
+                r = (int)(rg + (st >> 16));
                 x = (int)(st & 0xffffu);
                 read = ReadRef(R, R.read_off[r]);
                 L = R.read_len[r];
@@ -530,7 +542,7 @@ __global__ void __launch_bounds__(256) k_smem_global(SmemIn R, FmDev F, int min_
 {
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= n_ids) return;                     // at most n_ids lanes take reads: list slots g < n_ids
-    smem_lanes<WRITE>(R, F, min_len, n_ids, ids, lists + g * cap, cap, W);
+    smem_lanes<WRITE>(R, F, min_len, n_ids, ids, lists + g * cap, W);
 }
 
 // first[r] = the records before read r, first[n] = their number: sums of tiles of
@@ -625,30 +637,29 @@ int grid_for(int64_t n, int per_block, int sms, int per_sm)
 
 int64_t smem_tiles(int64_t n_reads) { return (n_reads + kFirstTile - 1) / kFirstTile; }
 
-cudaError_t launch_smem_store(const SmemIn &R, const FmDev &F, int min_len, const SmemWork &W, int64_t chunk,
+cudaError_t launch_smem_clear(int64_t n_reads, const SmemWork &W, cudaStream_t st)
+{
+    const cudaError_t e = cudaMemsetAsync(W.count, 0, sizeof(int64_t) * (size_t)n_reads, st);
+    return e != cudaSuccess ? e : cudaMemsetAsync(W.totals, 0, sizeof(SmemTotals), st);
+}
+
+cudaError_t launch_smem_store(const SmemIn &R, const FmDev &F, int min_len, const SmemWork &W, int64_t r0, int64_t nr,
                               cudaStream_t st, int sms)
 {
-    if (R.n_reads <= 0) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(W.count, 0, sizeof(int64_t) * (size_t)R.n_reads, st);
+    const cudaError_t e = cudaMemsetAsync(W.ctr, 0, sizeof(SmemCounters), st);
     if (e != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(W.totals, 0, sizeof(SmemTotals), st)) != cudaSuccess) return e;
-    const int64_t groups = (R.n_reads + 31) / 32;
+    const int64_t ng = (nr + 31) / 32;
     constexpr int warps = kSmemThreads / 32;
-    for (int64_t g0 = 0; g0 < groups; g0 += chunk) {
-        const int64_t ng = groups - g0 < chunk ? groups - g0 : chunk;
-        if ((e = cudaMemsetAsync(W.next, 0, 4, st)) != cudaSuccess) return e;
-        k_smem_scan<<<(unsigned)((ng + warps - 1) / warps), kSmemThreads, 0, st>>>(R, F, min_len, W, g0, ng);
-        k_smem_store<<<grid_for(ng, warps, sms, kSmemBlocksPerSm), kSmemThreads, 0, st>>>(R, F, min_len, W, g0, ng);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    k_smem_scan<<<(unsigned)((ng + warps - 1) / warps), kSmemThreads, 0, st>>>(R, F, min_len, W, r0, nr);
+    k_smem_store<<<grid_for(ng, warps, sms, kSmemBlocksPerSm), kSmemThreads, 0, st>>>(R, F, min_len, W, r0, ng);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_smem_global(bool write, const SmemIn &R, const FmDev &F, int min_len, const SmemWork &W,
                                const int32_t *ids, int64_t n_ids, BiIv *lists, int cap, cudaStream_t st, int sms)
 {
     if (n_ids <= 0) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(W.next, 0, 4, st);
+    cudaError_t e = cudaMemsetAsync(W.ctr, 0, sizeof(SmemCounters), st);
     if (e != cudaSuccess) return e;
     const int blocks = grid_for(n_ids, 256, sms, 8);
     if (write) k_smem_global<true><<<blocks, 256, 0, st>>>(R, F, min_len, W, ids, n_ids, lists, cap);

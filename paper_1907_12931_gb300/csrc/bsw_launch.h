@@ -243,9 +243,10 @@ constexpr int kSmemThreads = 128, kListCap = 24, kSmemBlocksPerSm = 7;
 // bases keep 16 (155 949 reads of 250 bp: 3.3 ms against 4.5 a call; 200 000 of 151 bp hold at
 // most 8).
 constexpr int kSmemKeep = 8, kSmemKeepLong = 16, kSmemKeepLen = 160;
-// Search starts a group of 32 reads of at most lmax bases has room for.  Past a
-// sequencing error a search reaches about 13 bases, so twice that many fit.
-constexpr int smem_starts_cap(int lmax) { return 32 * (4 + lmax / 6); }
+// Search starts there is room for per read of len bases (a group of 32 reads
+// shares its reads' room).  Past a sequencing error a search reaches about 13
+// bases, so twice that many fit.
+__host__ __device__ constexpr int smem_room(int len) { return 4 + len / 6; }
 
 // What the host reads back of a search.
 struct SmemTotals {
@@ -253,29 +254,41 @@ struct SmemTotals {
     int64_t records;
 };
 
+// Where the search starts of a group of 32 reads lie in W.starts, and how many.
+struct SmemGroup {
+    int64_t at;
+    int32_t n, pad;
+};
+
+// Counters of a launch: the next group or read to take, the entries of W.starts
+// given to groups.
+struct SmemCounters {
+    unsigned long long used;
+    uint32_t next, pad;
+};
+
 // Buffers of one SMEM search.  Store mode: count[r] (2^40 or more, and r once in
 // ovf_list[totals->overflows++], when a list of the read exceeds kListCap or its
-// starts the group's room) and up to
-// keep matches {start, length, k, s} at scratch[r * keep].  Write
-// mode: records at out[first[r]].  next: the launch's read counter (zeroed by the launchers).
+// starts the group's room) and up to keep matches {start, length, k, s} at
+// scratch[r * keep].  Write mode: records at out[first[r]].
 struct SmemWork {
     int64_t *count;
     uint4 *scratch;
     int64_t *first;          // [n_reads + 1]
     bsw_smem_t *out;
-    uint32_t *next;
+    SmemCounters *ctr;       // zeroed by the launchers
     SmemTotals *totals;
     int32_t *ovf_list;
     int32_t *many;           // reads with more than keep records (totals->many)
     int64_t *tile_sum;       // [smem_tiles(n_reads)]
-    uint32_t *starts;        // [groups of 32 reads][starts_cap] search starts: start | lane << 16
-    uint32_t *n_starts;      // [groups]: the starts noted
-    int32_t starts_cap;
+    uint32_t *starts;        // the round's search starts: start | lane << 16
+    SmemGroup *group;        // [groups of 32 reads of the round]
     int32_t keep;            // kSmemKeep or kSmemKeepLong
 };
-// W.starts and W.n_starts hold `chunk` groups; the reads are searched in as
-// many rounds as that takes.
-cudaError_t launch_smem_store(const SmemIn &R, const FmDev &F, int min_len, const SmemWork &W, int64_t chunk,
+// Counts and totals of all reads to zero, before the first round.
+cudaError_t launch_smem_clear(int64_t n_reads, const SmemWork &W, cudaStream_t st);
+// One round: reads [r0, r0 + nr), whose smem_room W.starts holds.
+cudaError_t launch_smem_store(const SmemIn &R, const FmDev &F, int min_len, const SmemWork &W, int64_t r0, int64_t nr,
                               cudaStream_t st, int sms);
 // The reads ids[0..n_ids) in store or write mode with lists in `lists` (cap
 // entries per lane, n_ids lanes at most).

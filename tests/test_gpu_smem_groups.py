@@ -3,8 +3,9 @@
 k_smem_scan takes groups of 32 reads and notes the searches' starts,
 k_smem_store works them off, in as many rounds as the budget's room for starts
 takes.  Cases: read counts around a group, empty and one-base reads, reads
-unrelated to the text (a start every dozen bases), and a budget that holds one
-group of starts at a time.
+unrelated to the text (a start every dozen bases), budgets that hold the starts
+of a few reads at a time, one long read among short ones, and starts given up
+for other calls.
 """
 import numpy as np
 import pytest
@@ -62,27 +63,102 @@ def test_group_edges(bsw, n):
             assert search(bsw, ctx, reads, min_len) == expected(ref, reads, min_len)
 
 
+def rounds_of(bsw, call):
+    """Rounds of a search: as many of its launches as an injected failure can skip."""
+    for k in range(1, 1000):
+        assert bsw.bsw_fault_inject("launch:%d" % k) == bsw.BSW_OK
+        try:
+            call()
+        except bsw.BswError as e:
+            assert e.code == bsw.BSW_ECUDA
+            continue
+        finally:
+            bsw.bsw_fault_inject(None)
+        return k
+
+
 def test_rounds_under_a_tight_budget(bsw):
-    """The smallest budgets that hold the reads and their records also hold the
-    search, group by group."""
+    """Budgets down to the least that holds the reads and their records: the
+    search then runs in rounds, with reads on both sides of a round's end in one
+    group of 32.  No read needs lists or has more records than are kept."""
     rng = np.random.default_rng(8)
     ref = rng.integers(0, 4, 2000).astype(np.uint8)
-    reads = make_reads(rng, ref, 300, 600)
-    want = expected(ref, reads, 12)
-    done = 0
-    for budget in range(200_000, 2_000_000, 25_000):
+    reads = make_reads(rng, ref, 301, 600)
+    want = expected(ref, reads, 50)
+    assert 0 < max(len(r) for r in want) <= 8
+    seen = set()
+    for budget in list(range(60_000, 200_000, 3_000)) + [1 << 22]:
         with bsw.Context(W.Params(), budget) as ctx:
-            ctx.fm_build(ref)
             try:
-                got = search(bsw, ctx, reads, 12)
+                ctx.fm_build(ref)
+                got = search(bsw, ctx, reads, 50)
             except bsw.BswError as e:
-                assert e.code == bsw.BSW_EBUDGET and done == 0
+                assert e.code == bsw.BSW_EBUDGET and not seen
                 continue
-        assert got == want
-        done += 1
-        if done == 12:
-            break
-    assert done >= 3
+            assert got == want
+            seen.add(rounds_of(bsw, lambda: search(bsw, ctx, reads, 50)))
+            assert search(bsw, ctx, reads, 50) == want
+    assert 1 in seen and 2 in seen and max(seen) >= 5, seen
+
+
+def long_among_short():
+    """20 000 reads of 60 bases, 40 of them with some ten records, and one of 32 768."""
+    rng = np.random.default_rng(5)
+    ref = rng.integers(0, 4, 50_000).astype(np.uint8)
+    reads = [ref[p:p + 60].copy() for p in rng.integers(0, 49_000, 20_000)]
+    for x in reads[:40]:
+        x[::6] = (x[::6] + 1) % 4
+    one = rng.integers(0, 4, 32768).astype(np.uint8)
+    one[:30000] = ref[:30000]
+    return ref, reads[:7000] + [one] + reads[7000:]
+
+
+def test_one_long_read_among_short_ones(bsw):
+    """The long read takes room for its own starts, not for every group's, and
+    the lists of the reads with many records find their room: 40 MB hold the
+    call, as they hold the reads, their records and 41 lists."""
+    ref, reads = long_among_short()
+    with bsw.Context(W.Params(), 1 << 30) as ctx:
+        ctx.fm_build(ref)
+        want = search(bsw, ctx, reads, 4)
+    few = [k for k in range(len(reads)) if k % 500 == 0 and len(reads[k]) < 100] + [3, 39]
+    assert [want[k] for k in few] == expected(ref, [reads[k] for k in few], 4)
+    assert sum(len(r) > 8 for r in want) >= 40
+    with bsw.Context(W.Params(), 40 << 20) as ctx:
+        ctx.fm_build(ref)
+        for _ in range(2):                                         # the second with the first's lists still held
+            assert search(bsw, ctx, reads, 4) == want
+
+
+def test_starts_are_given_up(bsw):
+    """Where an allocation is refused, the starts an earlier search left make
+    room for it; a search does with half the starts where theirs is refused."""
+    rng = np.random.default_rng(10)
+    ref = rng.integers(0, 4, 2000).astype(np.uint8)
+    reads = make_reads(rng, ref, 200, 130)
+    want = expected(ref, reads, 12)
+    sa = np.arange(3_000_000, dtype=np.int32)
+    with bsw.Context(W.Params(), 1 << 30) as ctx:
+        ctx.fm_build(ref)
+        assert search(bsw, ctx, reads, 12) == want
+        try:
+            bsw.bsw_fault_inject("alloc")
+            ctx.sal_set_index(sa[:1_000_000])                      # refused once: the starts go, and it passes
+            bsw.bsw_fault_inject("alloc")
+            with pytest.raises(bsw.BswError) as e:                 # nothing left to give up
+                ctx.sal_set_index(sa)
+            assert e.value.code == bsw.BSW_ENOMEM
+        finally:
+            bsw.bsw_fault_inject(None)
+        assert search(bsw, ctx, reads, 12) == want
+    with bsw.Context(W.Params(), 1 << 30) as ctx:
+        ctx.fm_build(ref)
+        try:
+            bsw.bsw_fault_inject("alloc:1")                        # the staging buffer passes, the starts do not
+            assert search(bsw, ctx, reads, 12) == want
+        finally:
+            bsw.bsw_fault_inject(None)
+        assert rounds_of(bsw, lambda: search(bsw, ctx, reads, 12)) == 1
 
 
 @pytest.mark.parametrize("lmax,budget", [(160, 1 << 30), (161, 1 << 30), (300, 1 << 30), (300, 3 << 20)])
