@@ -144,10 +144,13 @@ __device__ __forceinline__ uint32_t first_row(const FmDev &F, int c)
     return c < 2 ? (c == 0 ? F.C[0] : F.C[1]) : c == 2 ? F.C[2] : c == 3 ? F.C[3] : F.C[4];
 }
 
-// Whether a search can start at base c (4: N): the text holds it.
-__device__ __forceinline__ bool in_text(const FmDev &F, int c)
+// The bases a search can start at, bit c for base c: those the text holds (no N).
+__device__ __forceinline__ uint32_t text_bases(const FmDev &F)
 {
-    return c < 4 && first_row(F, c + 1) != first_row(F, c);
+    uint32_t m = 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) m |= (uint32_t)(F.C[c + 1] != F.C[c]) << c;
+    return m;
 }
 
 // A read of the batch: its packed bases (a read starts on a byte) and its base
@@ -193,6 +196,7 @@ __device__ void smem_lanes(const SmemIn &R, const FmDev &F, int min_len, int64_t
                            BiIv *list, const SmemWork &W)
 {
     enum { kRead, kCall, kBack, kEnd, kFwd, kBwd };
+    const uint32_t held = text_bases(F);
     int state = kRead;
     int r = 0, n = 0, call0 = 0;
     int64_t o = 0;
@@ -226,7 +230,7 @@ __device__ void smem_lanes(const SmemIn &R, const FmDev &F, int min_len, int64_t
                     continue;
                 }
                 const int c0 = base_at(x);
-                if (!in_text(F, c0)) {
+                if (!((held >> c0) & 1u)) {
                     ++x;
                     continue;
                 }
@@ -364,6 +368,7 @@ __global__ void __launch_bounds__(kSmemThreads) k_smem_scan(SmemIn R, FmDev F, i
     if (lane == 0) part = atomicAdd(&W.ctr->used, (unsigned long long)room);
     part = __shfl_sync(kAll, part, 0);
     uint32_t *starts = W.starts + part;
+    const uint32_t held = text_bases(F);
     uint32_t quad = 0;
     int i = 0, x = -1, n = 0;                // the next base; the search's start (-1: none); starts noted
     uint32_t vk = 0, vl = 0, vs = 0;         // the match X[x..i), its rows and those of its reverse complement
@@ -375,7 +380,7 @@ __global__ void __launch_bounds__(kSmemThreads) k_smem_scan(SmemIn R, FmDev F, i
         const uint32_t s2 = c < 4 ? u.size : 0u;
         const bool ends = i < L && x >= 0 && s2 == 0;
         if (ends && x == 0) emit_match(W, min_len, r, 0, i, vk, vs);
-        const bool starts_here = i < L && (x < 0 || ends) && in_text(F, c);
+        const bool starts_here = i < L && (x < 0 || ends) && ((held >> c) & 1u);
         if (starts_here) {
             vk = first_row(F, c);
             vl = first_row(F, 3 - c);
