@@ -33,9 +33,14 @@ constexpr int kNumCounters = kNumClass + 3;
 // so the persistent kernels take the longest work first.  The 8-bit bins also
 // split each query length by h0 (16 buckets of 16, largest first): a pair's
 // band starts about h0 columns wide, so 32 pairs of one bucket keep the lanes
-// of a warp on similar trip counts.
+// of a warp on similar trip counts.  The 16-bit bins hold the pairs with score
+// bounds past kRp16Top apart from the others within each class's lengths: the
+// class kernel runs the former one row at a time and the latter two, and a warp
+// with both pays for both (1 M pairs of 250 bp reads with match 10, half of them
+// past it: 10.63 ms in bins by length alone, 6.13 so).
 constexpr int kU8H0Buckets = 16;
-constexpr int kBinU8 = 0, kBinI16 = 256 * kU8H0Buckets, kBinW16 = kBinI16 + 256, kBinW32 = kBinW16 + 640,
+constexpr int kRp16Top = 2047;
+constexpr int kBinU8 = 0, kBinI16 = 256 * kU8H0Buckets, kBinW16 = kBinI16 + 2 * 256, kBinW32 = kBinW16 + 640,
               kNumBins = kBinW32 + 640;
 
 // Status bits written by the kernels.

@@ -37,6 +37,14 @@ constexpr int kNeg = -(1 << 29);
 
 // ------------------------------------------------------------------ bucketing
 
+// Bin of a 16-bit pair: of the lengths of its class (kI16Nmax) first the pairs
+// past kRp16Top, then the others.
+__device__ __forceinline__ int i16_bin(int n, long long bound)
+{
+    const int top = n > 128 ? 256 : n > 64 ? 128 : n > 32 ? 64 : 32;
+    return kBinI16 + 2 * (kShortMax - top) + (bound > kRp16Top ? 0 : max(top / 2, 32)) + (top - n);
+}
+
 __device__ __forceinline__ int pick_bin(int n, long long bound, uint32_t flags, int short_max, int h0, bool has_n)
 {
     const int u8 = kBinU8 + (kShortMax - n) * kU8H0Buckets + (kU8H0Buckets - 1 - min(h0 >> 4, kU8H0Buckets - 1));
@@ -53,9 +61,9 @@ __device__ __forceinline__ int pick_bin(int n, long long bound, uint32_t flags, 
     // kShortMax on the per-thread kernels whatever the plan says.
     if (n <= ((flags & (BSW_FORCE_I8 | BSW_FORCE_I16)) ? kShortMax : short_max)) {
         if (flags & BSW_FORCE_I8) return u8;
-        if (flags & BSW_FORCE_I16) return kBinI16 + (kShortMax - n);
+        if (flags & BSW_FORCE_I16) return i16_bin(n, bound);
         if (bound <= 255) return u8;
-        if (bound <= 32767) return kBinI16 + (kShortMax - n);
+        if (bound <= 32767) return i16_bin(n, bound);
         return kBinW32 + rank;
     }
     return bound <= 32767 ? kBinW16 + rank : kBinW32 + rank;
@@ -668,7 +676,6 @@ struct RpLane8 {
 // beside the slots, a nibble each, eight to a word, so that one permute gives
 // a row's scores of four columns.  A block's keys are H * 8 + step in 16 bits
 // and join the row's 32-bit keys (H * 512 + column) once a block.
-constexpr int kRp16Top = 2047;
 __host__ __device__ constexpr int rp16_words(int nmax) { return nmax + 1 + nmax / 8 + 1; }
 
 template <bool SYM>
@@ -2262,7 +2269,7 @@ bool make_plan(int short_max, uint32_t u8_mask, uint32_t i16_mask, bool packed, 
     // - n / 64): the block-per-pair class takes those of n >= cta_min
     b[kClsCTA] = kBinW16;
     b[kClsW16] = kBinW16 + (cta_min ? 640 - (cta_min >> 6) : 0);
-    for (int c = 11; c >= 9; --c) b[c] = ((i16_mask >> (c - 8)) & 1u) ? kBinI16 + kShortMax - kI16Nmax[c - 8] : b[c + 1];
+    for (int c = 11; c >= 9; --c) b[c] = ((i16_mask >> (c - 8)) & 1u) ? kBinI16 + 2 * (kShortMax - kI16Nmax[c - 8]) : b[c + 1];
     b[kClsW32] = kBinW32;
     b[kNumClass] = kNumBins;
     *out = L;
@@ -2511,7 +2518,7 @@ bool class_live(int c, const Plan &L, uint32_t flags)
     if (L.cls.b[c] == L.cls.b[c + 1]) return false;
     if (flags & (BSW_FORCE_I8 | BSW_FORCE_I16)) return true;
     const int nmin = u8 ? kShortMax - (L.cls.b[c + 1] - kBinU8) / kU8H0Buckets + 1   // the class's shortest query
-                        : kShortMax - (L.cls.b[c + 1] - kBinI16) + 1;
+                        : kShortMax - (L.cls.b[c + 1] - kBinI16) / 2 + 1;
     return nmin <= L.short_max;
 }
 

@@ -5,8 +5,11 @@ packed instruction, the others one row at a time.  The cases sit at that line
 (h0 + match * min(n, m) at 2046 to 2049), at the code words' and blocks' edges
 (query lengths around multiples of 8, and each class's bound), and at row
 counts of one to nine.  Every comparison is bit-exact on all six result fields
-and the cell count.
+and the cell count.  A batch with bounds on both sides of the line costs no more
+than one with all of them past it.
 """
+import time
+
 import numpy as np
 import pytest
 
@@ -57,3 +60,38 @@ def test_edges(bsw, sc, w, zd):
         got, gc = run(bsw, wl, flags=flags, device=True)
         assert_same(got, ref, "16-bit rows %s w=%d flags %d" % (sc, w, flags))
         assert gc == int(cells.sum())
+
+
+@pytest.mark.parametrize("bounds", [0xf, 0x1, 0x5])
+def test_bounds_on_both_sides(bsw, bounds):
+    """Every second pair past the line, in all classes and with classes of
+    several lengths merged: no warp runs both ways, so the batch takes less than
+    one of the slower kind alone (half a kind each: about 0.75 of it; in warps
+    that mix them 1.4)."""
+    rng = np.random.default_rng(bounds)
+    m1 = 4096
+    qs, ts = zip(*[near_copy(rng, int(n), int(n) + 60) for n in rng.choice([30, 60, 120, 121, 250], m1)])
+    k = np.arange(160_000)
+    params = W.Params(W.Scoring(8, 32, 48, 8, 48, 8), w=100, zdrop=800, end_bonus=40)
+    ms = {}
+    for name, past in (("both", k % 2 == 0), ("past", k >= 0)):
+        hs = [int((2100 if p else 2047) - 8 * len(qs[j % m1])) for j, p in zip(k, past)]
+        assert min(hs) >= 0
+        wl = W.from_lists([qs[j % m1] for j in k], [ts[j % m1] for j in k], hs, params, align=4)
+        if name == "both":
+            ref, cells, _ = oracle.extend_batch(wl, nthreads=NTH)
+        with bsw.Context(params, 4 << 30) as ctx:
+            ctx.set_plan(bsw.make_plan(i16_bounds=bounds))
+            db = bsw.DeviceBatch(bsw.HostBatch(wl))
+            t = []
+            for _ in range(8):
+                ctx.sync()
+                t0 = time.perf_counter()
+                ctx.extend_device(db)
+                ctx.sync()
+                t.append(1e3 * (time.perf_counter() - t0))
+            if name == "both":
+                assert_same(db.out.cpu().numpy(), ref, "both sides, bounds %x" % bounds)
+                assert int(db.cells.item()) == int(cells.sum())
+        ms[name] = min(t[2:])
+    assert ms["both"] < ms["past"], ms
