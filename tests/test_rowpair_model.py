@@ -1,13 +1,15 @@
-"""The 8-bit row-pair scheme against the oracle, on the host (no GPU).
+"""The row-pair scheme against the oracle, on the host (no GPU).
 
-`rowpair_model.extend` restates the kernel's two-rows-per-instruction pass
-bit by bit (packed instructions emulated on 32-bit words).  These tests pin
-the scheme itself: every result field and the cell count equal the oracle's
-for random pairs under symmetric and split gap costs, match scores 1 to 3
-and bands of 0 to 100 columns; for pairs whose rows read slots past the
-previous row's end (the oracle counts those reads); and for every row count
-from 1 to 9.  The GPU tests in `test_gpu_rowpair.py` check the kernel on the
-same kinds of input.
+`rowpair_model.extend` restates the kernels' two-rows-per-instruction pass bit
+by bit (packed instructions emulated on 32-bit words), for the 8-bit lanes
+without and with N bases and for the 16-bit lanes.  These tests pin the scheme
+itself: every result field and the cell count equal the oracle's for random
+pairs under symmetric and split gap costs, match scores 1 to 3 and bands of 0
+to 100 columns (16-bit lanes: match scores up to 127 and bounds up to 2047);
+for pairs whose rows read slots past the previous row's end (the oracle counts
+those reads); and for every row count from 1 to 9.  The GPU tests in
+`test_gpu_rowpair.py`, `test_gpu_nbase.py` and `test_gpu_rows16.py` check the
+kernels on the same kinds of input.
 """
 import numpy as np
 import pytest
@@ -36,10 +38,12 @@ def random_case(rng):
     return params, q.astype(np.uint8), t.astype(np.uint8), h0
 
 
-def same(params, q, t, h0, what):
+def same(params, q, t, h0, what, lanes=({}, {"nm": True}, {"lane": rowpair_model.Lane16})):
+    """On each lane: 8-bit without N codes and with them (none in the pair), 16-bit."""
     ref, cells, stale = oracle.extend_one(params, q, t, h0)
-    got, gc = rowpair_model.extend(params, q, t, h0)
-    assert got == ref and gc == cells, (what, len(q), len(t), h0, params, ref, cells, got, gc)
+    for lane in lanes:
+        got, gc = rowpair_model.extend(params, q, t, h0, **lane)
+        assert got == ref and gc == cells, (what, lane, len(q), len(t), h0, params, ref, cells, got, gc)
     return stale
 
 
@@ -97,18 +101,62 @@ def test_row_counts():
                     same(W.Params(W.Scoring(), w=w, zdrop=1, end_bonus=5), q, t, h0, "rows")
 
 
+@pytest.mark.parametrize("seed", range(2))
+def test_n_bases(seed):
+    """N in queries and targets, on the 8-bit lane that takes them."""
+    rng = np.random.default_rng(950 + seed)
+    done = 0
+    while done < 200:
+        params, q, t, h0 = random_case(rng)
+        if h0 is None:
+            continue
+        q[rng.random(len(q)) < rng.choice([0.0, 0.02, 0.3])] = 4
+        t[rng.random(len(t)) < rng.choice([0.0, 0.02, 0.3])] = 4
+        same(params, q, t, h0, "N %d" % seed, lanes=({"nm": True},))
+        done += 1
+
+
+@pytest.mark.parametrize("seed", range(4))
+def test_scores_past_eight_bits(seed):
+    """The 16-bit lane at bounds from 256 to 2047, under match scores up to 127
+    and gap costs past the largest score."""
+    rng = np.random.default_rng(970 + seed)
+    done = 0
+    while done < 150:
+        a = int(rng.choice([1, 2, 5, 20, 60, 127]))
+        n, m = int(rng.integers(1, 61)), int(rng.integers(1, 91))
+        left = 2047 - a * min(n, m)
+        if left < 0:
+            continue
+        h0 = left if done % 3 == 0 else int(rng.integers(0, left + 1))
+        q = rng.integers(0, 4, n).astype(np.uint8)
+        t = np.where(rng.random(m) < 0.9, np.resize(q, m), rng.integers(0, 4, m)).astype(np.uint8)
+        od, ed = int(rng.choice([0, 6, 200, 3000])), int(rng.choice([1, 2, 40]))
+        oi, ei = (od, ed) if rng.random() < 0.5 else (int(rng.choice([0, 9, 2500])), int(rng.choice([1, 7])))
+        params = W.Params(W.Scoring(a, int(rng.choice([1, 4, 40, 128])), od, ed, oi, ei),
+                          w=int(rng.choice([0, 1, 3, 10, 100])), zdrop=int(rng.choice([0, 20, 500])), end_bonus=5)
+        same(params, q, t, h0, "bound %d" % (2047 - left + h0), lanes=({"lane": rowpair_model.Lane16},))
+        done += 1
+
+
 def test_packed_helpers():
     """The emulated packed instructions act on each 16-bit half alone."""
     m = rowpair_model
     for lo_a, hi_a, lo_b, hi_b, lo_c, hi_c in [(5, -3, 2, 7, 4, -9), (-100, 200, 50, -50, 0, 0), (255, 0, 3, -4, 256, 1)]:
         a, b, c = m.pack(lo_a, hi_a), m.pack(lo_b, hi_b), m.pack(lo_c, hi_c)
         assert m.viaddmin_s16x2(a, b, c) == m.pack(min(lo_a + lo_b, lo_c), min(hi_a + hi_b, hi_c))
-        assert m.viaddmax_s16x2_relu(a, b, c) == m.pack(max(lo_a + lo_b, lo_c, 0), max(hi_a + hi_b, hi_c, 0))
+        assert m.viaddmax_s16x2(a, b, c) == m.pack(max(lo_a + lo_b, lo_c), max(hi_a + hi_b, hi_c))
         assert m.vimax3_s16x2(a, b, c) == m.pack(max(lo_a, lo_b, lo_c), max(hi_a, hi_b, hi_c))
-    # the selector of slot j gives s(t_i, q_j) low and s(t_{i+1}, q_{j-1}) high, sign-extended
-    prof0, prof1 = 0x01FCFCFC, 0xFCFC01FC        # row i: base 3 matches; row i+1: base 1
-    for qj in range(4):
-        for qjm in range(4):
-            sel = qj * 0x11 + qjm * 0x1100 + 0xC480
-            r = m.prmt(prof0, prof1, sel)
-            assert m.lo16(r) == (1 if qj == 3 else -4) and m.hi16(r) == (1 if qjm == 1 else -4)
+        assert m.sub_sat_h2(a, m.pack(7, 11)) == m.pack(max(0, lo_a - 7), max(0, hi_a - 11))
+    # the selector of slot j gives s(t_i, q_j) high and s(t_{i+1}, q_{j-1}) low, sign-extended
+    params = W.Params(W.Scoring(1, 4, 6, 1, 6, 1))
+    for nm in (False, True):
+        for qj in range(5 if nm else 4):
+            for qjm in range(5 if nm else 4):
+                lane = m.Lane8(params.scoring, [qjm, qj], 0, nm)
+                lane.rows(3, 1)
+                r = lane.scores(lane.S[1])
+                assert m.hi16(r) == (-1 if qj == 4 else 1 if qj == 3 else -4)
+                assert m.lo16(r) == (-1 if qjm == 4 else 1 if qjm == 1 else -4)
+                assert lane.score0(1) == m.hi16(r)
+                assert lane.score1(0) == m.lo16(r)
