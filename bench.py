@@ -40,9 +40,13 @@ import numpy as np  # noqa: E402
 LANE_OPS_PER_CLK_PER_SM = 128
 METRIC = "BSW GCUPS on 1 GB300 (batched vs plain kernel, bit-exact); p50/p99 serve latency"
 # DRAM bytes read + written per launch of a workload's dominant kernel, from
-# one ncu capture of the current kernel: (workload, class) -> (bytes, source);
-# others report null.  Empty until the row-pair kernels' launch is captured alone.
-MEASURED_TRAFFIC = {}
+# one ncu capture of the current kernel: (workload, class, cells of the launch)
+# -> (bytes, source); others report null.
+MEASURED_TRAFFIC = {
+    ("read250", "k_rows2 n<=128", 6_394_426_909): (48_376_320 + 345_856,
+                                                   "ncu dram__bytes_read.sum + dram__bytes_write.sum of the "
+                                                   "dominant launch, profiles/k_rows2_read250.md"),
+}
 
 SECONDARY = ("read151", "long10k")
 
@@ -225,17 +229,17 @@ def class_of(q_len, t_len, h0, match, plan):
 
 
 def class_kernel(c, plan, scoring):
-    """Label of class c under the plan: "k_inter" (one pair per thread; the kernels are k_rows2 and
-    k_rows2_16) or "k_inter2" with the class's bound, or the warp or block kernel's name."""
+    """Label of class c under the plan: the kernel, and for the per-thread ones (k_rows2, k_rows2_16, two
+    pairs per thread k_inter2) the class's longest query."""
     packable = (scoring.match + min(scoring.mismatch, 255 - scoring.match)
                 + max(min(scoring.o_del + scoring.e_del, 255), min(scoring.o_ins + scoring.e_ins, 255)) <= 256)
     if c < 8:
         nm = U8_NMAX[c]
         if plan.packed and nm <= 128 and packable:
             return "k_inter2<%d>" % (128 if nm > 64 else 64 if nm > 32 else 32)
-        return "k_inter<%d,u8>" % nm
+        return "k_rows2 n<=%d" % nm
     if c < 12:
-        return "k_inter<%d,i16>" % I16_NMAX[c - 8]
+        return "k_rows2_16 n<=%d" % I16_NMAX[c - 8]
     if c == 12:
         return "k_cta<8,s16>"
     if c == 13 and getattr(plan, "warp_x2", 0) and scoring.match <= 3:
@@ -747,7 +751,7 @@ def measure(bsw, args, name, dist, stream, local, world, rank, headline):
     gcups_plain = total_cells / (ms_plain * 1e-3) / 1e9
     sms = torch.cuda.get_device_properties(local).multi_processor_count
     roof = dominant_leg(bsw, ctx, wl, plan, stream, dist, steps, clk["sm_mhz"], sms)
-    traffic = MEASURED_TRAFFIC.get((name, roof["kernel_name"])) if args.pairs is None or not headline else None
+    traffic = MEASURED_TRAFFIC.get((name, roof["kernel_name"], roof["cells_per_launch"]))
     roof["traffic"] = traffic[0] if traffic else None
     roof["traffic_source"] = traffic[1] if traffic else None
     roof["dram_gbs"] = round(traffic[0] / (roof["launch_ms"] * 1e-3) / 1e9, 1) if traffic else None
