@@ -849,11 +849,9 @@ __device__ unsigned long long xr_pair(const Batch &B, const Params &P, int p, ui
     return S.ncell;
 }
 
-// Shared memory per warp of k_warp_x2: the ring or the scores and row copy.
-__host__ __device__ constexpr int x2_warp_bytes(int lg)
-{
-    return lg > 0 && x2_ring_words(lg) * 8 > kXrBytes ? (x2_ring_words(lg) * 8 + 63) / 64 * 64 : kXrBytes;
-}
+// A warp's shared memory in k_warp_x2 holds the scores and row copy, or the ring,
+// whose largest is smaller.
+static_assert(x2_ring_words(12) * 8 <= kXrBytes && (size_t)kX2Warps * x2_ring_words(13) * 8 > kRingSmemMax);
 
 // Persistent kernel over a class list: pairs whose score bound or band the
 // packed kernel does not hold go to the 32-bit re-run list.  A 10 kbp pair
@@ -869,7 +867,7 @@ __global__ void __launch_bounds__(kX2Warps * 32, 3) k_warp_x2(Batch B, Params P,
 {
     extern __shared__ __align__(64) uint4 x2_mem[];
     const int lane = threadIdx.x & 31, wj = threadIdx.x >> 5;
-    char *mem = reinterpret_cast<char *>(x2_mem) + wj * x2_warp_bytes(ring_log2);
+    char *mem = reinterpret_cast<char *>(x2_mem) + wj * kXrBytes;
     uint2 *ring = reinterpret_cast<uint2 *>(mem);
     const X2K K = x2_consts(P);
     const long long limit = 1ll << (15 - K.zsh);
@@ -896,6 +894,8 @@ __global__ void __launch_bounds__(kX2Warps * 32, 3) k_warp_x2(Batch B, Params P,
         const long long bound = (long long)B.h0[p] + (long long)P.a * min(n, m);
         if (bound < limit && xr_fits(P, n, B.h0[p], wb)) {
             cells += xr_pair<SYM>(B, P, p, sh_addr(mem), K);
+        // the host launches k_warp where no ring fits (0); without the test this
+        // kernel takes 149 registers instead of 146 and 0.5% longer
         } else if (ring_log2 > 0 && x2_ring_cols(wb) <= (1 << ring_log2) && bound < limit) {
             cells += x2_pair<SYM>(B, P, p, ring, x2_ring_cols(wb) - 1, K);
         } else if (lane == 0) {
@@ -971,10 +971,9 @@ cudaError_t prepare_x2(int sms)
     if ((e = cudaFuncSetAttribute(k_plain_x2<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingSmemMax)) !=
         cudaSuccess)
         return e;
-    // resident blocks for the ring of a w = 500 band (the long-query workload's)
     int nb = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_warp_x2<true>, kX2Warps * 32,
-                                                           (size_t)kX2Warps * x2_warp_bytes(10))) != cudaSuccess)
+                                                           (size_t)kX2Warps * kXrBytes)) != cudaSuccess)
         return e;
     // 3 blocks (12 warps) per SM, the class kernel's launch bound: its scores
     // and rows take 74 KB of shared memory a block, and a 10 kbp pair runs most
@@ -996,7 +995,7 @@ cudaError_t launch_x2(const Batch &B, const Params &P, const Work &W, int cls, c
 {
     if (sms * g_x2_blocks > 65535) return cudaErrorInvalidConfiguration;   // 16-bit stratum fields
     const int lg = x2_ring_log2(P);
-    const size_t smem = (size_t)kX2Warps * x2_warp_bytes(lg);
+    const size_t smem = (size_t)kX2Warps * kXrBytes;
     const bool sym = P.o_del == P.o_ins && P.e_del == P.e_ins;
     if (sym) k_warp_x2<true><<<sms * g_x2_blocks, kX2Warps * 32, smem, st>>>(B, P, W, cls, lg);
     else k_warp_x2<false><<<sms * g_x2_blocks, kX2Warps * 32, smem, st>>>(B, P, W, cls, lg);
