@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(kSmemThreads) k_smem_scan(SmemIn R, FmDev F, i
 // A pass of the main loop makes one extension on every lane, forward or
 // backward; a forward one is a backward one of revcomp(P), see smem_lanes.
 // Bound by the lookups (random 32-byte reads, mostly L2 hits).  200 k reads of
-// 151 bp against a 32 Mbp text: k_smem_scan 0.29 ms and this kernel 1.12 ms, with
+// 151 bp against a 32 Mbp text: k_smem_scan 0.28 ms and this kernel 1.10 ms, with
 // 25 and 18 of 32 lanes active; one kernel with a lane per read, lists of 16-byte
 // entries and two loads per bucket took 1.84 ms at 15 lanes.  24 matches a lane
 // and 7 blocks an SM run as fast as 28 and 6, 1% faster than 20 and 8.

@@ -7,7 +7,7 @@
 // thread that feed each other (so nothing folds), SM cycles from clock64().
 // Output: one JSON object per line.  It is a measurement program, not part of
 // the library; build it with
-//   nvcc -O3 -gencode arch=compute_103a,code=sm_103a -o _build/int_rates int_rates.cu
+//   nvcc -O3 -gencode arch=compute_103a,code=sm_103a -o _build/int_rates profiles/int_rates.cu
 #include <cuda_runtime.h>
 #include <cstdio>
 #include <vector>
